@@ -35,7 +35,9 @@
 //        in the buffer;
 //     c. the buffer is written as whole 16-byte chunks, consecutive lanes
 //        on consecutive chunks of one view row (one large L2 write per view
-//        row instead of one per block row).
+//        row instead of one per block row).  Rows that do not start on a
+//        16-byte boundary go out as the destination's aligned chunks, shifted
+//        into place (store_row_unaligned).
 // Reconstructions are 16-bit values plus a bias of 2^14, two to a word (the
 // loader refuses streams whose values could leave that range).  Every stored
 // block of the strip is decoded once.
@@ -120,8 +122,8 @@ struct Args {
     uint32_t par_base;       // BFS position (or top index) of the first parent of a view
     uint32_t n_par;          // parents of views
     uint32_t nlx, nloc, W, H;
-    uint32_t vec16;          // a strip's view rows go out as whole 16-byte chunks (16-byte aligned output; RGB: W % 16 == 0, packed: W % 4 == 0)
-    uint32_t vec4;           // where they cannot, as 4-byte words (4-byte aligned output; RGB also W % 4 == 0)
+    uint32_t pitch;          // pixels from one output row to the next: W, or the packed views' padded row (packed_pitch)
+    uint32_t vec16;          // every view row of a strip starts on a 16-byte boundary (16-byte aligned output; RGB: W % 16 == 0; packed: always)
     uint32_t pmax;           // largest number of stored blocks in the records of one strip
     uint32_t n_units;        // ceil(S / kUnit)
     uint32_t node_smem;      // the node table is cached in shared memory
@@ -134,9 +136,11 @@ struct Args {
 
 template <bool kPacked>
 __host__ __device__ constexpr uint32_t row_words() { return kPacked ? 4u : 3u; }
-// one warp's output buffer, in 16-byte chunks: kUnit views x 4 rows x kNL locations x row_words
+// one warp's output buffer, in 16-byte chunks: kUnit views x 4 rows x kNL
+// locations x row_words, between one chunk of padding on each side (the
+// unaligned row writer reads up to 16 bytes around a row)
 template <bool kPacked>
-__host__ __device__ constexpr uint32_t obuf_words() { return kUnit * 4 * kNL * row_words<kPacked>() / 4; }
+__host__ __device__ constexpr uint32_t obuf_words() { return kUnit * 4 * kNL * row_words<kPacked>() / 4 + 2; }
 
 struct Smem {
     uint32_t *slots;   // [warp][kWSlots + 1][8]  decoded blocks, biased pairs; slot kZeroSlot is zero
@@ -301,7 +305,51 @@ __device__ __forceinline__ void row_to_rgb(const uint2 y, const uint2 co, const 
 template <bool kPacked>
 __device__ __forceinline__ uint8_t *out_px(const Args &a, uint32_t ov, uint32_t y, uint32_t x)
 {
-    return a.out + (((size_t)ov * a.H + y) * a.W + x) * (kPacked ? 4u : 3u);
+    return a.out + (((size_t)ov * a.H + y) * a.pitch + x) * (kPacked ? 4u : 3u);
+}
+
+// Bytes [0, len) of a strip row (`src`, word-aligned shared memory with a
+// chunk of readable padding on each side) to `row`, whatever its alignment:
+// lane `ch` of eight takes the 16-byte aligned chunk ch of the destination,
+// which begins at source byte 16 ch - (row & 15); five words funnel-shifted to
+// four make it, and only the first and last chunk of the row, shared with the
+// neighbouring strips, go out as words and bytes.  len <= 112.
+//
+// What bounds it: instruction issue (about 25 instructions for up to 512
+// bytes; the edges another 40).  The 15 x 15 x 625 x 434 decode takes 0.250 ms
+// with it; with single bytes or 4-byte words, each placed by divisions by the
+// row length, it took 0.695 ms.
+__device__ __forceinline__ void store_row_unaligned(uint8_t *row, const uint32_t *src, uint32_t len, uint32_t ch)
+{
+    const int b0 = (int)(16u * ch) - (int)((uintptr_t)row & 15u);
+    const int lo = max(0, -b0), hi = min(16, (int)len - b0);   // this chunk's bytes
+    if (hi <= lo)
+        return;
+    const uint32_t *w = src + (b0 >> 2);
+    const uint32_t sh = 8u * ((uint32_t)b0 & 3u);
+    const uint32_t x0 = w[0], x1 = w[1], x2 = w[2], x3 = w[3], x4 = w[4];
+    const uint32_t y0 = __funnelshift_r(x0, x1, sh), y1 = __funnelshift_r(x1, x2, sh);
+    const uint32_t y2 = __funnelshift_r(x2, x3, sh), y3 = __funnelshift_r(x3, x4, sh);
+    uint8_t *p = row + b0;
+    if (hi - lo == 16) {
+        *reinterpret_cast<uint4 *>(p) = make_uint4(y0, y1, y2, y3);
+        return;
+    }
+    uint32_t *p4 = reinterpret_cast<uint32_t *>(p);
+    if (lo <= 0 && hi >= 4)
+        p4[0] = y0;
+    if (lo <= 4 && hi >= 8)
+        p4[1] = y1;
+    if (lo <= 8 && hi >= 12)
+        p4[2] = y2;
+    if (lo <= 12 && hi >= 16)
+        p4[3] = y3;
+    const uint8_t *sb = reinterpret_cast<const uint8_t *>(src) + b0;
+    const int up = (lo + 3) & ~3;
+    for (int j = lo; j < min(hi, up); j++)
+        p[j] = sb[j];
+    for (int j = max(hi & ~3, up); j < hi; j++)
+        p[j] = sb[j];
 }
 
 template <bool kPacked, typename OffT>
@@ -527,9 +575,10 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     const uint32_t nrows = min(4u, a.H - by * 4);
     constexpr uint32_t BPP = kPacked ? 4u : 3u;     // output bytes per pixel
     constexpr uint32_t CH = kNL * 4 * BPP / 16;     // 16-byte chunks per view row of the strip
-    uint4 *wbuf = reinterpret_cast<uint4 *>(m.obuf) + warp * obuf_words<kPacked>();
-    // a strip row written as whole chunks: every location present and 16-byte aligned rows
-    const bool whole = a.vec16 && nl == (uint32_t)kNL;
+    uint4 *wbuf = reinterpret_cast<uint4 *>(m.obuf) + warp * obuf_words<kPacked>() + 1;
+    // a strip row written as whole chunks: 16-byte aligned rows with room for
+    // the whole strip (a packed row is padded to whole strips)
+    const bool whole = a.vec16 && bx0 * 4 + kNL * 4 <= a.pitch;
     // otherwise the strip row's bytes (the image may end inside the strip)
     const uint32_t piece = min(nl * 4u, a.W - bx0 * 4u) * BPP;
     for (;;) {
@@ -667,8 +716,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
             L0 = L1;
         }
         // (c) write the unit's rows: consecutive lanes, consecutive chunks of one view row
+        const size_t row_bytes = (size_t)a.pitch * BPP;
         if (whole) {
-            const size_t row_bytes = (size_t)a.W * BPP;
 #pragma unroll
             for (uint32_t vv = 0; vv < (uint32_t)kUnit; vv++) {
                 uint8_t *o = reinterpret_cast<uint8_t *>(
@@ -676,23 +725,17 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
                 if (((sel >> (ub + vv)) & 1u) && f_act && f_rr < nrows && o)
                     reinterpret_cast<uint4 *>(o + f_rr * row_bytes)[f_c] = wbuf[vv * 4 * CH + lane];
             }
-        } else {
-            // the right edge of the image, or rows not 16-byte aligned: 4-byte
-            // words where the rows allow, else bytes
-            const uint8_t *bb = reinterpret_cast<const uint8_t *>(wbuf);
-            const uint32_t unit = (a.vec4 && piece % 4 == 0) ? 4u : 1u, per = piece / unit;
-            for (uint32_t i = lane; i < kUnit * 4 * per; i += 32) {
-                const uint32_t vv = i / (4 * per), rr = (i / per) & 3u, k = i % per;
-                const uint32_t view = ((sel >> (ub + vv)) & 1u) ? node_view(nodes[w * 32 + ub + vv]) : 0u;
-                const uint32_t ov = ((sel >> (ub + vv)) & 1u) ? (a.slot_of ? __ldg(a.slot_of + view) : view) : 0u;
-                if (((sel >> (ub + vv)) & 1u) && rr < nrows && RLFC_DBG_INDEX_OK(a.dbg, ov, a.n_out)) {
-                    uint8_t *dst = out_px<kPacked>(a, ov, by * 4 + rr, bx0 * 4) + k * unit;
-                    const uint8_t *src = bb + (vv * 4 + rr) * (kNL * 4 * BPP) + k * unit;
-                    if (unit == 4)
-                        *reinterpret_cast<uint32_t *>(dst) = *reinterpret_cast<const uint32_t *>(src);
-                    else
-                        *dst = *src;
-                }
+        } else if (!kPacked) {
+            // rows not 16-byte aligned, or the right edge of the image: lane =
+            // (row, 16-byte chunk of the destination)
+            const uint32_t rr = (uint32_t)lane >> 3, ch = (uint32_t)lane & 7u;
+#pragma unroll 2
+            for (uint32_t vv = 0; vv < (uint32_t)kUnit; vv++) {
+                uint8_t *o = reinterpret_cast<uint8_t *>(
+                    __shfl_sync(kFullMask, reinterpret_cast<unsigned long long>(out_v), vv));
+                if (((sel >> (ub + vv)) & 1u) && rr < nrows && o)
+                    store_row_unaligned(o + rr * row_bytes, reinterpret_cast<const uint32_t *>(wbuf + (vv * 4 + rr) * CH),
+                                        piece, ch);
             }
         }
         __syncwarp();
@@ -733,13 +776,8 @@ int launch_decode(const rlfc_stream *s, uint8_t *d_out, const uint8_t *needed, c
         a.par_base = t.n_int - n1;
         a.n_par = n1;
     }
-    if (kPacked) {
-        a.vec16 = ((uintptr_t)d_out & 15u) == 0 && (a.W & 3u) == 0;
-        a.vec4 = ((uintptr_t)d_out & 3u) == 0;
-    } else {
-        a.vec16 = ((uintptr_t)d_out & 15u) == 0 && (a.W & 15u) == 0;
-        a.vec4 = ((uintptr_t)d_out & 3u) == 0 && (a.W & 3u) == 0;
-    }
+    a.pitch = kPacked ? packed_pitch(a.W) : a.W;
+    a.vec16 = ((uintptr_t)d_out & 15u) == 0 && (kPacked || (a.W & 15u) == 0);
     a.pmax = std::max<uint32_t>(s->max_strip_present, 1);
     a.n_units = (t.S + kUnit - 1) / kUnit;
     a.node_smem = t.S <= kNodeSmemMax;

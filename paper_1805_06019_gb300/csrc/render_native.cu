@@ -65,7 +65,8 @@ struct Args {
     const float *disp;
     float *out;
     uint8_t *out8;             // when set, 8-bit RGB goes here instead of out
-    const uint32_t *decoded;   // packed RGB views [slot][H][W] decoded for this call, or null
+    const uint32_t *decoded;   // packed RGB views [slot][H][pitch] decoded for this call, or null
+    uint32_t pitch;            // pixels per row of a packed view
     const uint32_t *slot_of;   // with decoded views: the slot of each view
     uint32_t U, V, W, H, n;
     uint32_t tiles_x, cells_u;
@@ -455,8 +456,8 @@ __global__ void __launch_bounds__(kThreads, kDecoded ? 4 : 3) render_native_kern
                         locate(rb, kb, r_b);
                     const Window &wa = s_win[ka];
                     const Window &wb = s_win[kb];
-                    const uint32_t *sa = a.decoded + ((size_t)a.slot_of[nview[ka]] * a.H + min(max(wa.wy0 + ra, 0), (int)a.H - 1)) * a.W;
-                    const uint32_t *sb = a.decoded + ((size_t)a.slot_of[nview[kb]] * a.H + min(max(wb.wy0 + r_b, 0), (int)a.H - 1)) * a.W;
+                    const uint32_t *sa = a.decoded + ((size_t)a.slot_of[nview[ka]] * a.H + min(max(wa.wy0 + ra, 0), (int)a.H - 1)) * a.pitch;
+                    const uint32_t *sb = a.decoded + ((size_t)a.slot_of[nview[kb]] * a.H + min(max(wb.wy0 + r_b, 0), (int)a.H - 1)) * a.pitch;
                     uint32_t va0, va1, va2, vb0 = 0u, vb1 = 0u, vb2 = 0u;
                     va0 = lane < wa.WX ? __ldg(sa + min(max(wa.wx0 + lane, 0), (int)a.W - 1)) : 0u;
                     va1 = lane + 32 < wa.WX ? __ldg(sa + min(max(wa.wx0 + lane + 32, 0), (int)a.W - 1)) : 0u;
@@ -836,7 +837,8 @@ int launch_render_native(const rlfc_stream *s, const float *d_uv, const float *d
     a.decoded = nullptr;
     a.slot_of = nullptr;
     void *scratch = nullptr;
-    const size_t view_words = (size_t)a.W * a.H;
+    a.pitch = packed_pitch(a.W);
+    const size_t view_words = (size_t)a.pitch * a.H;
     const size_t mask_bytes = (a.sv.n_views + 255) / 256 * 256;
     const size_t slot_bytes = (4ull * a.sv.n_views + 255) / 256 * 256;
     const size_t n_slots = std::min<size_t>(a.sv.n_views, 4ull * n);

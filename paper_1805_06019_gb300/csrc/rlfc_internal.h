@@ -91,10 +91,16 @@ int build_tables(uint32_t L, const std::vector<uint32_t> &cnt,
 int cuda_fail(cudaError_t e, const char *what);
 
 int launch_decode_all(const rlfc_stream *s, uint8_t *d_out, cudaStream_t st);
-// every view the mask marks (all when null), as packed RGB words [view][H][W]
+// Pixels from one row of a packed view to the next: whole decode strips, so
+// that every strip row is written as aligned 16-byte chunks.
+inline uint32_t packed_pitch(uint32_t W)
+{
+    const uint32_t strip = 4 * kDecodeStrip;
+    return (W + strip - 1) / strip * strip;
+}
 // Packed RGB words of the views `needed` marks, view v into slot slot_of[v]
-// of d_out ([slot][H][W], n_slots slots); with needed null, every view v into
-// slot v.
+// of d_out ([slot][H][packed_pitch(W)], n_slots slots, 16-byte aligned); with
+// needed null, every view v into slot v.
 int launch_decode_packed(const rlfc_stream *s, uint32_t *d_out, const uint8_t *needed, const uint32_t *slot_of,
                          uint32_t n_slots, cudaStream_t st);
 // Largest |value| of any stored block of the stream, decoded (synchronous).
