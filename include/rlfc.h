@@ -164,9 +164,11 @@ RLFC_API int rlfc_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, co
  * views they need into a transient device buffer (stream-ordered
  * allocation on cuda_stream, released before the call's work completes:
  * 4 * H * (W rounded up to 32) bytes per needed view, at most min(views, 4n)
- * of them); if that
- * allocation fails the call decodes on demand instead.  Results do not
- * depend on the path or on the other views of the call.
+ * of them, and about 200 bytes per camera); if that allocation fails the
+ * call decodes on demand instead.  The loaded stream's own memory pool keeps
+ * what its calls used for the next ones, up to the packed size of all its
+ * views and at most 512 MiB, until rlfc_free_stream.  Results do not depend
+ * on the path or on the other views of the call.
  * Errors: RLFC_E_INVALID_ARG, RLFC_E_RANGE, RLFC_E_UNSUPPORTED, RLFC_E_CUDA.
  */
 RLFC_API int rlfc_render_views(const rlfc_stream *s, const float *d_uv, const float *d_disp,

@@ -732,60 +732,6 @@ __global__ void __launch_bounds__(kListThreads) list_cells_kernel(const Args a, 
         *count = total;
 }
 
-// Numbers the marked views 0, 1, ... in view order (one CTA; at most 16383
-// views, 16 per thread): slot_of[v] for a marked view v.
-__global__ void __launch_bounds__(kListThreads) assign_slots_kernel(const uint8_t *needed, uint32_t n_views,
-                                                                    uint32_t *slot_of)
-{
-    __shared__ uint32_t s_warp[kListThreads / 32];
-    const uint32_t per = (n_views + kListThreads - 1) / kListThreads;
-    const uint32_t v0 = threadIdx.x * per, v1 = min(n_views, v0 + per);
-    uint32_t cnt = 0;
-    for (uint32_t v = v0; v < v1; v++)
-        cnt += needed[v] != 0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t incl = cnt;
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= d)
-            incl += y;
-    }
-    if (lane == 31)
-        s_warp[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t w = s_warp[lane];
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, w, d);
-            if (lane >= d)
-                w += y;
-        }
-        s_warp[lane] = w;
-    }
-    __syncthreads();
-    uint32_t at = incl - cnt + (warp ? s_warp[warp - 1] : 0u);
-    for (uint32_t v = v0; v < v1; v++)
-        if (needed[v])
-            slot_of[v] = at++;
-}
-
-// Marks the neighbour views that each camera blends with a non-zero weight.
-__global__ void mark_needed_kernel(const Args a, uint8_t *needed)
-{
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= a.n)
-        return;
-    int ci, cj;
-    float w[4];
-    Shift sh[4];
-    view_params(a, r, ci, cj, w, sh);
-    for (int k = 0; k < 4; k++) {
-        const int i = a.U == 1 ? 0 : ci + (k & 1), j = a.V == 1 ? 0 : cj + (k >> 1);
-        if (w[k] != 0.0f)
-            needed[j * (int)a.U + i] = 1;
-    }
-}
-
 }  // namespace
 
 // Native-size rendering of n views; returns RLFC_E_UNSUPPORTED when the
@@ -829,35 +775,22 @@ int launch_render_native(const rlfc_stream *s, const float *d_uv, const float *d
     const uint32_t single = win1 + 4 * ((kTW + 7) / kBlock + 1) * ((kTH + 7) / kBlock + 1) * 3 * 2 * a.need_max;
     cudaError_t e;
 
-    // Batches of many views decode the views they need once into a transient
-    // packed-RGB buffer (stream-ordered allocation, freed on the same stream),
-    // one slot per needed view: a camera needs at most four views, so
-    // min(views, 4n) slots suffice.  Small batches decode block by block
-    // inside the render kernel.
+    if (n >= kDecodeFirstViews) {
+        const int rc = launch_render_windows(s, d_uv, d_disp, n, d_out, st, d_out8);
+        if (rc != RLFC_E_UNSUPPORTED)
+            return rc;
+    }
     a.decoded = nullptr;
     a.slot_of = nullptr;
-    void *scratch = nullptr;
-    a.pitch = packed_pitch(a.W);
-    const size_t view_words = (size_t)a.pitch * a.H;
-    const size_t mask_bytes = (a.sv.n_views + 255) / 256 * 256;
-    const size_t slot_bytes = (4ull * a.sv.n_views + 255) / 256 * 256;
-    const size_t n_slots = std::min<size_t>(a.sv.n_views, 4ull * n);
-    bool first = n >= kDecodeFirstViews && win1 <= kSmemDecoded;
-    if (first && cudaMallocAsync(&scratch, mask_bytes + slot_bytes + 4 * view_words * n_slots, st) != cudaSuccess) {
-        cudaGetLastError();   // a failed stream-ordered allocation only selects the other path
-        first = false;
-    }
-    if (!first && single > kSmemBytes)
+    if (single > kSmemBytes)
         return RLFC_E_UNSUPPORTED;
-    auto kern = first ? render_native_kernel<true> : render_native_kernel<false>;
-    const uint32_t smem = first ? kSmemDecoded : kSmemBytes;
+    auto kern = render_native_kernel<false>;
+    const uint32_t smem = kSmemBytes;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem)) != cudaSuccess) {
-        if (scratch)
-            cudaFreeAsync(scratch, st);
         return cuda_fail(e, "render_native: launch configuration");
     }
     dim3 grid(a.n_tiles, n_cells);
@@ -871,7 +804,7 @@ int launch_render_native(const rlfc_stream *s, const float *d_uv, const float *d
         // cell, so list the occupied cells and run persistent CTAs over their
         // tiles only (list and count in stream-ordered scratch)
         grid = dim3(resident);
-        if ((e = cudaMallocAsync(&cells, 4ull * (n_cells + 1), st)) != cudaSuccess) {
+        if ((e = scratch_alloc(s, (void **)&cells, 4ull * (n_cells + 1), st)) != cudaSuccess) {
             rc = cuda_fail(e, "render_native: cell list");
         } else {
             a.cell_list = cells;
@@ -879,27 +812,11 @@ int launch_render_native(const rlfc_stream *s, const float *d_uv, const float *d
             { rlfc::TraceScope trace_("list_cells_kernel", st); list_cells_kernel<<<1, kListThreads, 0, st>>>(a, n_cells, cells, cells + n_cells); }
         }
     }
-    if (rc == RLFC_OK && first) {
-        uint8_t *needed = static_cast<uint8_t *>(scratch);
-        uint32_t *slot_of = reinterpret_cast<uint32_t *>(needed + mask_bytes);
-        uint32_t *decoded = reinterpret_cast<uint32_t *>(needed + mask_bytes + slot_bytes);
-        if ((e = cudaMemsetAsync(needed, 0, mask_bytes, st)) != cudaSuccess)
-            rc = cuda_fail(e, "render: clearing the view mask");
-        if (rc == RLFC_OK) {
-            { rlfc::TraceScope trace_("mark_needed_kernel", st); mark_needed_kernel<<<(n + 255) / 256, 256, 0, st>>>(a, needed); }
-            { rlfc::TraceScope trace_("assign_slots_kernel", st); assign_slots_kernel<<<1, kListThreads, 0, st>>>(needed, a.sv.n_views, slot_of); }
-            rc = launch_decode_packed(s, decoded, needed, slot_of, (uint32_t)n_slots, st);
-        }
-        a.decoded = decoded;
-        a.slot_of = slot_of;
-    }
     if (rc == RLFC_OK) {
         { rlfc::TraceScope trace_("render_native_kernel", st); kern<<<grid, kThreads, smem, st>>>(a); }
         if ((e = cudaGetLastError()) != cudaSuccess)
             rc = cuda_fail(e, "render_native launch");
     }
-    if (scratch)
-        cudaFreeAsync(scratch, st);
     if (cells)
         cudaFreeAsync(cells, st);
     return rc;

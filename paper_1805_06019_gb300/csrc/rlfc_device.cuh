@@ -194,12 +194,15 @@ __device__ __forceinline__ uint32_t ycocg_to_rgb24(int y, int co, int cg)
 // 8-bit output of a rendered value: floor(clamp(v, 0, 1) * 255 + 0.5), the
 // product and the sum each rounded on their own (never fused), so the result
 // equals that of the same float operations anywhere else.
-__device__ __forceinline__ uint8_t to_u8(float v)
+// In the low byte of the result (the bits above it are not cleared).
+__device__ __forceinline__ uint32_t u8_value(float v)
 {
-    // __saturatef clamps to [0, 1] (NaN to 0); the argument of the
-    // round-down conversion is at least 0.5, so it is the floor
-    return (uint8_t)__float2uint_rd(__fadd_rn(__fmul_rn(__saturatef(v), 255.0f), 0.5f));
+    // __saturatef clamps to [0, 1] (NaN to 0); a value in [0.5, 255.5] plus
+    // 2^23, rounded down, has its floor in the low byte (on the FMA pipe; the
+    // float to integer conversion runs at a quarter of its rate)
+    return __float_as_uint(__fadd_rd(__fadd_rn(__fmul_rn(__saturatef(v), 255.0f), 0.5f), 8388608.0f));
 }
+__device__ __forceinline__ uint8_t to_u8(float v) { return (uint8_t)u8_value(v); }
 
 // Store a rendered RGB pixel (pixel index px) as floats, or as 8 bits when
 // out8 is set.
