@@ -205,11 +205,12 @@ def _kernel_bytes(info, stream_read, n_views_lf, n_needed, n_render, out_w, out_
         # packed views it writes are the renderer's own intermediate)
         "decode_all_kernel<packed>": stream_read,
         # camera table read, one mask byte per view written
-        "mark_needed_kernel": 12 * n_render + n_views_lf,
+        "render_plan_kernel": 12 * n_render + n_views_lf,
         # float RGB written (the decoded views it reads are the renderer's
         # own intermediate, not bytes the method must move)
         "render_native_kernel": 12 * out_px,
-        "render_tiled_kernel": stream_read + 12 * out_px,
+        "render_sampled_kernel": 12 * out_px,
+        "render_demand_kernel": stream_read + 12 * out_px,
         "render_direct_kernel": stream_read + 12 * out_px,
     }
 

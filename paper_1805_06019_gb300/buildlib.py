@@ -12,7 +12,7 @@ LIB = os.path.join(BUILD, "librlfc.so")
 # debug build: the device bounds checks compiled in (RLFC_DEBUG, rlfc_debug_flags)
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(BUILD_DEBUG, "librlfc.so")
-SOURCES = ["rlfc_host.cu", "trace.cu", "decode_batch.cu", "server.cu", "decode_all.cu", "decode_blocks.cu", "render.cu", "render_native.cu", "render_windows.cu",
+SOURCES = ["rlfc_host.cu", "trace.cu", "decode_batch.cu", "server.cu", "decode_all.cu", "decode_blocks.cu", "render.cu", "render_demand.cu", "render_windows.cu",
            "encode.cu", "encode_no_alloc.cu", "mlp.cu"]
 HEADERS = ["rlfc_device.cuh", "rlfc_internal.h", "warp_decode.cuh", "pair_decode.cuh", "render_camera.cuh", "ks_device.cuh"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"

@@ -54,6 +54,7 @@ __device__ __forceinline__ uint32_t neighbour_view(const Grid &g, uint32_t ci, u
 struct Stencil {
     int ox, oy;       // integer part of the neighbour's shift
     float fx, fy;     // fractional part
+    float sx, sy;     // the shift
 };
 
 // The neighbours' blend weights and shifts for focus disparity d.
@@ -74,6 +75,35 @@ __device__ __forceinline__ void camera_stencils(const Grid &g, const CameraCell 
         st[k].oy = (int)fly;
         st[k].fx = sx - flx;
         st[k].fy = sy - fly;
+        st[k].sx = sx;
+        st[k].sy = sy;
+    }
+}
+
+// ray of an output pixel, bilinear taps along one axis with clamp-to-edge
+__device__ __forceinline__ float ray_s(uint32_t x, uint32_t W, uint32_t out_w)
+{
+    return ((float)x + 0.5f) * (float)W / (float)out_w - 0.5f;
+}
+__device__ __forceinline__ void taps(float xs, uint32_t W, int &xa, int &xb, float &fx)
+{
+    const float x0 = floorf(xs);
+    fx = xs - x0;
+    const int xi = (int)x0;
+    xa = min(max(xi, 0), (int)W - 1);
+    xb = min(max(xi + 1, 0), (int)W - 1);
+}
+
+// One neighbour's bilinear sample at any output size, weighted and added.
+__device__ __forceinline__ void sample_add(float w, float fx, float fy, uint32_t p00, uint32_t p10, uint32_t p01, uint32_t p11,
+                                           float acc[3])
+{
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const auto v = [c](uint32_t rgb) { return (float)((rgb >> (8 * c)) & 255u); };
+        const float top = (1.0f - fx) * v(p00) + fx * v(p10);
+        const float bot = (1.0f - fx) * v(p01) + fx * v(p11);
+        acc[c] += w * (((1.0f - fy) * top + fy * bot) / 255.0f);
     }
 }
 

@@ -1,6 +1,6 @@
-// New-view rendering at the views' own resolution for batches of cameras
-// (Section 3.6): the neighbour views the batch needs are decoded once, then
-// every camera is blended from them.
+// New-view rendering for batches of cameras (Section 3.6): the neighbour views
+// the batch needs are decoded once, then every camera is blended from them: at
+// the views' own resolution from shared windows, at others sample by sample.
 //
 // Every new camera (u, v) inside grid cell (i0, j0) blends the same four
 // neighbour views (i0, j0), (i0+1, j0), (i0, j0+1), (i0+1, j0+1), and at
@@ -13,7 +13,7 @@
 //     shifted windows fit shared memory, marks the views needed and numbers
 //     their slots;
 //  2. the needed views are decoded into packed RGB slots (decode_all.cu);
-//  3. render_windows_kernel: persistent CTAs take (group, 64 x 32 tile) items
+//  3. render_native_kernel: persistent CTAs take (group, 64 x 32 tile) items
 //     from a queue, fill one window of the tile per neighbour, and blend the
 //     group's cameras from the windows.
 #include <cuda_runtime.h>
@@ -344,7 +344,7 @@ __device__ __forceinline__ void blend_rows(const CamS &c, int pitch_quads, int r
 // per thread, direct stores and the cameras' parameters computed by every
 // tile, 1.15 ms.
 template <bool kU8>
-__global__ void __launch_bounds__(kThreads, 3) render_windows_kernel(const Args a)
+__global__ void __launch_bounds__(kThreads, 3) render_native_kernel(const Args a)
 {
     constexpr int kPix = kU8 ? 3 : 12, kRowWords = kTW * kPix / 4;   // output bytes per pixel, staged words per row
     __shared__ Window s_win[4];
@@ -507,14 +507,50 @@ __global__ void __launch_bounds__(kThreads, 3) render_windows_kernel(const Args 
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the staged rows are read before the CTA ends
 }
 
+// Any output size: a thread per output pixel samples the decoded views through
+// the caches.  What bounds it: instruction issue (about 350 instructions per
+// pixel for 16 samples, their weights and coordinates).
+constexpr int kSX = 32, kSY = 8;
+
+__global__ void __launch_bounds__(kSX * kSY) render_sampled_kernel(const Args a, const float *uv, const float *disp, uint32_t out_w,
+                                                                    uint32_t out_h, uint32_t tiles_x)
+{
+    const uint32_t n = blockIdx.y;
+    const uint32_t x = (blockIdx.x % tiles_x) * kSX + threadIdx.x % kSX, y = (blockIdx.x / tiles_x) * kSY + threadIdx.x / kSX;
+    if (x >= out_w || y >= out_h)
+        return;
+    CameraCell c;
+    camera_cell(a.grid, uv, n, c);
+    Stencil st[4];
+    float w[4];
+    camera_stencils(a.grid, c, disp[n], w, st);
+    const float s = ray_s(x, a.grid.W, out_w), t = ray_s(y, a.grid.H, out_h);
+    float acc[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        if (w[k] == 0.0f)
+            continue;
+        int xa, xb, ya, yb;
+        float fx, fy;
+        taps(s + st[k].sx, a.grid.W, xa, xb, fx);
+        taps(t + st[k].sy, a.grid.H, ya, yb, fy);
+        const uint32_t *v = a.decoded + (size_t)a.slot_of[neighbour_view(a.grid, c.ci, c.cj, k)] * a.grid.H * a.pitch;
+        const uint32_t *ra = v + (size_t)(uint32_t)ya * a.pitch, *rb = v + (size_t)(uint32_t)yb * a.pitch;
+        sample_add(w[k], fx, fy, __ldg(ra + xa), __ldg(ra + xb), __ldg(rb + xa), __ldg(rb + xb), acc);
+    }
+    store_rgb(a.out, a.out8, ((size_t)n * out_h + y) * out_w + x, acc[0], acc[1], acc[2]);
+}
+
 }  // namespace
 
-// Native-size rendering of n views from views decoded for the call; returns
-// RLFC_E_UNSUPPORTED when the scratch cannot be had (the caller decodes on
-// demand instead).
-int launch_render_windows(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t n, float *d_out,
-                          cudaStream_t st, uint8_t *d_out8)
+// Rendering of n views from views decoded for the call: planned, decoded into
+// slots, then blended (at native size from windows, at others by samples).
+// Returns RLFC_E_UNSUPPORTED when the scratch cannot be had (the caller
+// decodes on demand instead).
+int launch_render_decoded(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t out_w, uint32_t out_h, uint32_t n,
+                          float *d_out, cudaStream_t st, uint8_t *d_out8)
 {
+    const bool native = out_w == s->info.W && out_h == s->info.H;
     Plan p;
     Args a;
     p.grid = a.grid = make_grid(s->info.U, s->info.V, s->info.W, s->info.H);
@@ -522,7 +558,9 @@ int launch_render_windows(const rlfc_stream *s, const float *d_uv, const float *
     a.pitch = packed_pitch(s->info.W);
     a.tiles_x = (s->info.W + kTW - 1) / kTW;
     a.n_tiles = a.tiles_x * ((s->info.H + kTH - 1) / kTH);
-    if (n_views > 32u * kPlanThreads || (uint64_t)a.n_tiles * n >= (1ull << 32) - (1u << 20))
+    const uint32_t stiles_x = (out_w + kSX - 1) / kSX;
+    const uint64_t stiles = (uint64_t)stiles_x * ((out_h + kSY - 1) / kSY);
+    if (n_views > 32u * kPlanThreads || (uint64_t)a.n_tiles * n >= (1ull << 32) - (1u << 20) || stiles >= (1ull << 31))
         return RLFC_E_UNSUPPORTED;
     // one stream-ordered block: the plan, then a slot per needed view (a
     // camera needs at most four views, so min(views, 4n) slots suffice)
@@ -554,7 +592,7 @@ int launch_render_windows(const rlfc_stream *s, const float *d_uv, const float *
     a.out8 = d_out8;
     a.bulk = d_out8 ? ((uintptr_t)d_out8 & 15u) == 0 && s->info.W % 16 == 0 : ((uintptr_t)d_out & 15u) == 0 && s->info.W % 4 == 0;
     const uint32_t win_bytes = p.win_bytes = d_out8 ? kWinBytesU8 : kWinBytes;
-    auto kern = d_out8 ? render_windows_kernel<true> : render_windows_kernel<false>;
+    auto kern = d_out8 ? render_native_kernel<true> : render_native_kernel<false>;
     const uint32_t plan_smem = 4u * (n_cells + 1 + 2 * ((n_views + 31) / 32)) + 2u * n_cells;
     int sms = 0, per_sm = 0, rc = RLFC_OK;
     cudaError_t e;
@@ -572,9 +610,13 @@ int launch_render_windows(const rlfc_stream *s, const float *d_uv, const float *
         { TraceScope trace_("render_plan_kernel", st); render_plan_kernel<<<1, kPlanThreads, plan_smem, st>>>(p); }
         rc = launch_decode_packed(s, reinterpret_cast<uint32_t *>(scratch + at_dec), p.needed, p.slot_of, (uint32_t)n_slots, st);
     }
-    if (rc == RLFC_OK) {
+    if (rc == RLFC_OK && !native) {
+        { TraceScope trace_("render_sampled_kernel", st); render_sampled_kernel<<<dim3((uint32_t)stiles, n), kSX * kSY, 0, st>>>(a, d_uv, d_disp, out_w, out_h, stiles_x); }
+        if ((e = cudaGetLastError()) != cudaSuccess)
+            rc = cuda_fail(e, "render_sampled launch");
+    } else if (rc == RLFC_OK) {
         const uint32_t grid = (uint32_t)std::min<uint64_t>(resident, (uint64_t)a.n_tiles * n);
-        { TraceScope trace_("render_windows_kernel", st); kern<<<grid, kThreads, win_bytes, st>>>(a); }
+        { TraceScope trace_("render_native_kernel", st); kern<<<grid, kThreads, win_bytes, st>>>(a); }
         if ((e = cudaGetLastError()) != cudaSuccess)
             rc = cuda_fail(e, "render_windows launch");
     }

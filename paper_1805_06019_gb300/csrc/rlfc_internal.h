@@ -111,13 +111,13 @@ int launch_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, const uin
 // Stream-ordered scratch for one call, from the stream's own pool (released
 // with cudaFreeAsync).
 cudaError_t scratch_alloc(const rlfc_stream *s, void **p, size_t bytes, cudaStream_t st);
-// Batches of cameras at native size, blended from views decoded for the call;
-// RLFC_E_UNSUPPORTED when its scratch cannot be had.
-int launch_render_windows(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t n,
-                          float *d_out, cudaStream_t st, uint8_t *d_out8);
-// d_out8: when set, 8-bit RGB output instead of d_out
-int launch_render_native(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t n,
-                         float *d_out, cudaStream_t st, uint8_t *d_out8 = nullptr);
+// n views (d_out8: when set, 8-bit RGB instead of d_out) from views decoded
+// for the call, or decoded on demand tile by tile; RLFC_E_UNSUPPORTED when
+// the scratch (or the shared memory) for it cannot be had.
+int launch_render_decoded(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t out_w, uint32_t out_h,
+                          uint32_t n, float *d_out, cudaStream_t st, uint8_t *d_out8);
+int launch_render_demand(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t out_w, uint32_t out_h,
+                         uint32_t n, float *d_out, cudaStream_t st, uint8_t *d_out8);
 int launch_render(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t out_w,
                   uint32_t out_h, uint32_t n, float *d_out, cudaStream_t st, uint8_t *d_out8 = nullptr);
 // arena: when given, every device buffer of the encoder is carved from it

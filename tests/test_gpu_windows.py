@@ -32,6 +32,19 @@ def test_batches_do_not_change_a_view(W, H, spread):
     u8 = st.render(duv, dd, W, H, u8=True)
     parts = torch.cat([st.render(duv[i:i + 5].contiguous(), dd[i:i + 5].contiguous(), W, H) for i in range(0, n, 5)])
     assert torch.equal(whole, parts)
+    # decoded on demand, one camera and two at a time (footprints apart when
+    # the shifts are large)
+    ones = torch.cat([st.render(duv[i:i + 1].contiguous(), dd[i:i + 1].contiguous(), W, H) for i in range(20)])
+    twos = torch.cat([st.render(duv[i:i + 2].contiguous(), dd[i:i + 2].contiguous(), W, H) for i in range(0, 20, 2)])
+    assert torch.equal(whole[:20], ones) and torch.equal(whole[:20], twos)
+    # other sizes: the same from decoded views (as a large batch) and on demand
+    for w, h in ((W // 2 + 3, H // 3 + 1), (W + 17, 2 * H)):
+        reps = 1 + 450_000 // (n * W * H)
+        many = st.render(duv.repeat(reps, 1), dd.repeat(reps), w, h)
+        few = torch.cat([st.render(duv[i:i + 2].contiguous(), dd[i:i + 2].contiguous(), w, h) for i in range(0, 20, 2)])
+        assert torch.equal(many[:20], few)
+        want = oracle.render_view(ref, U, V, float(uv[7, 0]), float(uv[7, 1]), float(d[7]), w, h)
+        assert np.abs(few[7].cpu().numpy() - want).max() <= 1e-3
     # an output off the 16-byte boundary, in both formats
     buf = torch.full((whole.numel() + 8,), -1.0, device="cuda")
     st.render(duv, dd, W, H, out=buf[1:1 + whole.numel()].view(whole.shape))
