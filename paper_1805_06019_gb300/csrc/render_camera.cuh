@@ -94,6 +94,18 @@ __device__ __forceinline__ void taps(float xs, uint32_t W, int &xa, int &xb, flo
     xb = min(max(xi + 1, 0), (int)W - 1);
 }
 
+// x / 255, correctly rounded, for x = 0 and normal x whose quotient is
+// normal: 1/255 as the sum of two floats (Brisebarre, Muller and Raina,
+// "Accelerating correctly rounded floating-point division when the divisor is
+// known in advance", 2004; checked for every mantissa).  Two instructions
+// instead of a division, twelve times a pixel: the sampled renderer takes 79
+// instead of 89 us for eight 800 x 600 views.
+__device__ __forceinline__ float div255(float x)
+{
+    constexpr float hi = 1.0f / 255.0f, lo = (float)(1.0 / 255.0 - (double)hi);
+    return fmaf(x, hi, x * lo);
+}
+
 // One neighbour's bilinear sample at any output size, weighted and added.
 __device__ __forceinline__ void sample_add(float w, float fx, float fy, uint32_t p00, uint32_t p10, uint32_t p01, uint32_t p11,
                                            float acc[3])
@@ -103,7 +115,7 @@ __device__ __forceinline__ void sample_add(float w, float fx, float fy, uint32_t
         const auto v = [c](uint32_t rgb) { return (float)((rgb >> (8 * c)) & 255u); };
         const float top = (1.0f - fx) * v(p00) + fx * v(p10);
         const float bot = (1.0f - fx) * v(p01) + fx * v(p11);
-        acc[c] += w * (((1.0f - fy) * top + fy * bot) / 255.0f);
+        acc[c] += w * div255((1.0f - fy) * top + fy * bot);
     }
 }
 
