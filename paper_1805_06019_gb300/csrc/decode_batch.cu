@@ -10,17 +10,24 @@
 //      contiguous in the stream) into its shared-memory slice, or has them
 //      copied there ahead of time (cp.async) while it serves the previous
 //      location;
-//   2. parses each record once: presence-mask popcount prefixes, then the
-//      closed-form payload length of every stored block from its 5-bit mode,
-//      turned into payload bit offsets by a warp scan;
-//   3. for up to kSlots requests at a time: seeds int32 accumulators with the
-//      top-RKV block, lists the stored ancestor blocks (request, channel,
-//      level) with a ballot compaction, decodes them one thread per block
-//      with the sequential bit reader and adds (min + u) 2^(q + s) into the
-//      accumulators, converts YCoCg-R to clamped RGB and writes 48 bytes per
-//      request.
+//   2. parses the three records once, side by side: presence-mask popcount
+//      prefixes, then the closed-form payload length of every stored block
+//      from its 5-bit mode, turned into payload bit offsets by a warp scan;
+//   3. for up to sixteen requests at a time: seeds accumulators (biased 16-bit
+//      pairs, pair_decode.cuh) with the top-RKV block, lists the stored
+//      ancestor blocks (request, channel, level) with a ballot compaction,
+//      decodes them one thread per block with the pair decoder and adds them
+//      into the accumulators (a packed add is exact modulo 2^32, so the order
+//      does not matter), then a thread per block row converts to RGB and the
+//      48 bytes of a request go out as three 16-byte stores.
 // The record gather (mask, headers, offsets) is paid once per location and
 // shared by every request there, which is the point of batching.
+//
+// What bounds it: the chain of dependent loads per location and instruction
+// issue (57 % of the slots, 27 of 32 lanes active); 10^6 requests on the 17 x
+// 17 x 1024^2 light field (133 MB stream) take 0.189 ms, 0.15 of them here.
+// With 32-bit accumulators, an atomic per value, the sequential bit reader,
+// eight requests a round and one record parsed after the other: 0.323 ms.
 #include <cuda_runtime.h>
 
 #include <cuda_pipeline.h>
@@ -28,18 +35,17 @@
 #include <algorithm>
 #include <new>
 
-#include "rlfc_device.cuh"
+#include "pair_decode.cuh"
 #include "rlfc_internal.h"
 
 namespace rlfc {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
-constexpr uint32_t kSlots = 8;          // requests of one location per round
+constexpr uint32_t kSlots = 16, kSlotsTight = 12;   // requests of one location per round; fewer where shared memory is short
+constexpr uint32_t kStaticLimit = 112;  // static shared memory that the limits of create and set_config count
 constexpr uint32_t kStageCap = 1024;    // words of records staged per warp at most
 constexpr uint32_t kBadRank = 0xFFFFFFFFu;
-
-__constant__ uint32_t c_modes[kNumModes] = RLFC_MODE_TABLE_INIT;
 
 __device__ __forceinline__ uint32_t scan_incl(uint32_t x, int lane)
 {
@@ -60,8 +66,7 @@ struct BinArgs {
     uint32_t *cnt;      // [nloc + 2]: counts, then bin starts; [nloc + 1] is the queue head,
                         // followed by the scan's per-chunk counts
     uint32_t *rank;     // [n]: position of the request inside its bin
-    uint32_t *sorted;   // [n]: request indices grouped by location
-    uint32_t *sorted_view;  // [n]: their views, in the same order
+    uint2 *sorted;      // [n]: requests grouped by location: index, view
     uint32_t n, n_views, nloc, aligned;
 };
 
@@ -167,9 +172,8 @@ __global__ void bin_scatter_kernel(const BinArgs a)
         return;
     const uint32_t rk = a.rank[r];
     if (rk != kBadRank) {
-        const uint32_t at = a.cnt[a.loc[r]] + rk;
-        a.sorted[at] = r;
-        a.sorted_view[at] = a.view[r];
+        // (one random 8-byte store per request: index and view side by side)
+        a.sorted[a.cnt[a.loc[r]] + rk] = make_uint2(r, a.view[r]);
     }
 }
 
@@ -178,199 +182,222 @@ struct DecArgs {
     const uint32_t *offsets;
     const int16_t *top;       // [n_top][nloc][48]
     const uint32_t *view_anc; // [n_views][kMaxLevels]
-    const uint32_t *req_view;
     const uint32_t *start;    // [nloc + 1] bin starts
-    const uint32_t *sorted;
-    const uint32_t *sorted_view;
+    const uint2 *sorted;
     uint8_t *out;
     uint32_t *queue;
-    uint32_t nloc, L, q, MW, level, pmax, locs_per_pop, stage, stage_words, warp_words, aligned;
-    uint32_t anc_words;       // view_anc words cached in shared memory (0: read it from global)
+    uint32_t nloc, L, q, MW, level, pmax, locs_per_pop, stage, stage_words, warp_words;
+    uint32_t slots;           // requests per round
+    uint32_t aligned;         // output alignment: 16, 4 or 1 bytes
+    uint32_t anc_views;       // views whose ancestors are cached in shared memory, 16 bits each (0: read them from global)
     uint32_t *dbg;            // debug builds: the stream's flag word
 };
 
 // Per-warp shared-memory words for a configuration (the CTA adds the cached
 // ancestor table after its warps' slices).
 // stage: 0 none, 1 one buffer, 2 two buffers (prefetch); each buffer holds
-// stage_words + 4 words.
-__host__ __device__ inline uint32_t warp_words_for(uint32_t MW, uint32_t pmax, uint32_t L, uint32_t stage,
-                                                   uint32_t stage_words)
+// stage_words + 4 words.  What a configuration may need (create and
+// set_config refuse larger ones) is at least what it uses with kSlotsTight.
+__host__ __device__ inline uint32_t warp_words_limit(uint32_t MW, uint32_t pmax, uint32_t L, uint32_t stage,
+                                                     uint32_t stage_words)
 {
-    const uint32_t w = 6 * MW + 3 * pmax + kSlots * 48 + 2 * kSlots + kSlots * 3 * (L - 1) + kSlots * 16 +
+    const uint32_t w = 6 * MW + 3 * pmax + 528 + 24 * (L - 1) + stage * (stage_words + 4);
+    return (w + 3u) & ~3u;
+}
+// masks and their prefixes, payload offsets, accumulators (8 pairs of each of
+// 3 channels per slot, at an odd pitch), request index and view, task list
+__host__ __device__ inline uint32_t warp_words_for(uint32_t MW, uint32_t pmax, uint32_t L, uint32_t stage, uint32_t stage_words,
+                                                   uint32_t off_bytes, uint32_t n)
+{
+    const uint32_t w = 6 * MW + (3 * pmax * off_bytes + 3) / 4 + 8 * (3 * n + 1) + 2 * n + 3 * n * (L - 1) +
                        stage * (stage_words + 4);
     return (w + 3u) & ~3u;
 }
 
-__global__ void __launch_bounds__(512) decode_binned_kernel(const DecArgs a)
+template <typename OffT>
+__global__ void __launch_bounds__(512, 2) decode_binned_kernel(const DecArgs a)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ uint32_t s_modes[kNumModes];
-    if (threadIdx.x < kNumModes)
-        s_modes[threadIdx.x] = c_modes[threadIdx.x];
+    __shared__ uint32_t s_mode[32];
+    __shared__ uint16_t s_dig[256 + 128];
+    if (threadIdx.x < 32)
+        s_mode[threadIdx.x] = g_tables.mode[threadIdx.x];
+    for (uint32_t i = threadIdx.x; i < (256 + 128) / 2; i += blockDim.x)
+        reinterpret_cast<uint32_t *>(s_dig)[i] = reinterpret_cast<const uint32_t *>(g_tables.dig)[i];
     // the ancestor table, shared by the CTA's warps when it is small
-    const uint32_t *view_anc = a.view_anc;
-    if (a.anc_words) {
-        uint32_t *s_anc = smem + (blockDim.x >> 5) * a.warp_words;
-        for (uint32_t i = threadIdx.x; i < a.anc_words; i += blockDim.x)
-            s_anc[i] = a.view_anc[i];
-        view_anc = s_anc;
-    }
+    uint16_t *s_anc = reinterpret_cast<uint16_t *>(smem + (blockDim.x >> 5) * a.warp_words);
+    for (uint32_t i = threadIdx.x; i < a.anc_views * kMaxLevels; i += blockDim.x)
+        s_anc[i] = (uint16_t)a.view_anc[i];
     __syncthreads();
+    const auto ancestor = [&](uint32_t view, uint32_t l) -> uint32_t {
+        return a.anc_views ? s_anc[view * kMaxLevels + l] : a.view_anc[view * kMaxLevels + l];
+    };
     const int lane = (int)(threadIdx.x & 31u);
+    const uint32_t pitch = 3 * a.slots + 1;
     uint32_t *s_mask = smem + (threadIdx.x >> 5) * a.warp_words;   // [3][MW]
-    uint32_t *s_mpre = s_mask + 3 * a.MW;                           // [3][MW] popcount before each word
-    uint32_t *s_off = s_mpre + 3 * a.MW;                            // [3][pmax] payload bit offsets
-    int32_t *s_acc = reinterpret_cast<int32_t *>(s_off + 3 * a.pmax);   // [kSlots][3][16]
-    uint32_t *s_req = reinterpret_cast<uint32_t *>(s_acc + kSlots * 48);
-    uint32_t *s_view = s_req + kSlots;
-    uint32_t *s_list = s_view + kSlots;                             // [kSlots * 3 * (L-1)]
-    uint32_t *s_rgb = s_list + kSlots * 3 * (a.L - 1);              // [kSlots][16]
-    uint32_t *s_stage = s_rgb + kSlots * 16;
+    uint32_t *s_mpre = s_mask + 3 * a.MW;                           // [3][MW] stored blocks in front of each word, records one after the other
+    uint32_t *s_acc = s_mpre + 3 * a.MW;                            // [8][pitch] pair j of (slot, channel)
+    uint32_t *s_list = s_acc + 8 * pitch;                           // [slots * 3 * (L-1)]
+    uint32_t *s_req = s_list + 3 * a.slots * (a.L - 1), *s_view = s_req + a.slots;
+    OffT *s_off = reinterpret_cast<OffT *>(s_view + a.slots);       // [3 pmax] payload bit offsets, records one after the other
+    uint32_t *s_stage = s_view + a.slots + (3 * a.pmax * (uint32_t)sizeof(OffT) + 3) / 4;
     const uint32_t nl = a.L - 1 - a.level;   // SRV levels added to the top RKV
     const uint32_t hdr0 = 32 * a.MW;
+    // (division of task numbers below 2^10 by 3 nl and nl)
+    const uint32_t inv3 = nl ? (65536u + 3 * nl - 1) / (3 * nl) : 0u, inv1 = nl ? (65536u + nl - 1) / nl : 0u;
 
     // One location: parse its three records (from `staged` when they were
     // copied to shared memory, else from the stream) and serve its requests.
     auto serve = [&](uint32_t loc, const uint32_t *staged) {
-        {
-            const uint32_t r0 = a.start[loc], r1 = a.start[loc + 1];
-            if (r0 == r1)
-                return;
-            const uint32_t o0 = a.offsets[3 * loc];
-            const uint32_t d1 = a.offsets[3 * loc + 1] - o0, d2 = a.offsets[3 * loc + 2] - o0;
-            const uint32_t span = a.offsets[3 * loc + 3] - o0;
-            const uint32_t *base = staged ? staged : a.records + o0;
-            if (!staged && a.stage == 1 && span <= a.stage_words) {
-                // the bit reader may touch one word past a record: copy two more
-                // (the stream carries zero padding after its last record)
-                for (uint32_t i = lane; i < span + 2; i += 32)
-                    s_stage[i] = base[i];
-                __syncwarp();
-                base = s_stage;
+        const uint32_t r0 = a.start[loc], r1 = a.start[loc + 1];
+        if (r0 == r1)
+            return;
+        const uint32_t o0 = a.offsets[3 * loc];
+        const uint32_t d1 = a.offsets[3 * loc + 1] - o0, d2 = a.offsets[3 * loc + 2] - o0;
+        const uint32_t span = a.offsets[3 * loc + 3] - o0;
+        const uint32_t *base = staged ? staged : a.records + o0;
+        if (!staged && a.stage == 1 && span <= a.stage_words) {
+            // the bit reader may touch two words past a record: copy them too
+            // (the stream carries zero padding after its last record)
+            for (uint32_t i = lane; i < span + 2; i += 32)
+                s_stage[i] = base[i];
+            __syncwarp();
+            base = s_stage;
+        }
+        const auto rec_of = [&](uint32_t c) { return base + (c == 0 ? 0u : (c == 1 ? d1 : d2)); };
+        // masks: a lane per (channel, word)
+        uint32_t total = 0, p1 = 0, p2 = 0;   // stored blocks; those in front of records 1 and 2
+        for (uint32_t w0 = 0; w0 < 3 * a.MW; w0 += 32) {
+            const uint32_t i = w0 + lane;
+            const uint32_t c = (i >= a.MW) + (i >= 2 * a.MW);
+            const uint32_t word = i < 3 * a.MW ? rec_of(c)[i - c * a.MW] : 0u;
+            const uint32_t cnt = __popc(word);
+            const uint32_t excl = total + scan_incl(cnt, lane) - cnt;
+            if (i < 3 * a.MW) {
+                s_mask[i] = word;
+                s_mpre[i] = excl;
             }
-            // parse the three records
-#pragma unroll
-            for (uint32_t c = 0; c < 3; c++) {
-                const uint32_t *rc = base + (c == 0 ? 0u : (c == 1 ? d1 : d2));
-                uint32_t total = 0;
-                for (uint32_t w0 = 0; w0 < a.MW; w0 += 32) {
-                    const uint32_t wi = w0 + lane;
-                    const uint32_t word = wi < a.MW ? rc[wi] : 0u;
-                    const uint32_t cnt = __popc(word);
-                    const uint32_t incl = scan_incl(cnt, lane);
-                    if (wi < a.MW) {
-                        s_mask[c * a.MW + wi] = word;
-                        s_mpre[c * a.MW + wi] = total + incl - cnt;
-                    }
-                    total += __shfl_sync(kFull, incl, 31);
+            if (a.MW - w0 < 32)
+                p1 = __shfl_sync(kFull, excl, a.MW - w0);
+            if (2 * a.MW - w0 < 32)
+                p2 = __shfl_sync(kFull, excl, 2 * a.MW - w0);
+            total = __shfl_sync(kFull, excl + cnt, 31);
+        }
+        // headers, record after record: payload offset of every stored block
+        // inside its record
+        const uint32_t pay0[3] = {hdr0 + kHdrBits * p1, hdr0 + kHdrBits * (p2 - p1), hdr0 + kHdrBits * (total - p2)};
+        uint32_t run = 0, g1 = 0, g2 = 0;     // payload bits so far; in front of records 1 and 2
+#pragma unroll 2
+        for (uint32_t h0 = 0; h0 < total; h0 += 32) {
+            const uint32_t i = h0 + lane;
+            const uint32_t c = (i >= p1) + (i >= p2), h = i - (c == 0 ? 0u : (c == 1 ? p1 : p2));
+            const uint32_t len = i < total ? mode_bits(s_mode[get_bits(rec_of(c), hdr0 + kHdrBits * h, 5)]) : 0u;
+            const uint32_t incl = scan_incl(len, lane), excl = run + incl - len;
+            if (p1 - h0 < 32)
+                g1 = __shfl_sync(kFull, excl, p1 - h0);
+            if (p2 - h0 < 32)
+                g2 = __shfl_sync(kFull, excl, p2 - h0);
+            if (i < total)
+                s_off[i] = (OffT)(pay0[0] * (c == 0) + (pay0[1] - g1) * (c == 1) + (pay0[2] - g2) * (c == 2) + excl);
+            run += __shfl_sync(kFull, incl, 31);
+        }
+        __syncwarp();
+        for (uint32_t j0 = r0; j0 < r1; j0 += a.slots) {
+            const uint32_t ns = min(a.slots, r1 - j0);
+            if ((uint32_t)lane < ns) {
+                const uint2 rq = a.sorted[j0 + lane];
+                s_req[lane] = rq.x;
+                s_view[lane] = rq.y;
+            }
+            __syncwarp();
+            // ReadBlock(RKV^n, BlkIdx): the accumulators start at the top RKV
+            // (96 bytes per slot, as six 16-byte loads)
+            for (uint32_t i = lane; i < ns * 6; i += 32) {
+                const uint32_t slot = (i * 10923u) >> 16, k = i - slot * 6;
+                const uint32_t top = ancestor(s_view[slot], a.L - 1);
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(a.top + ((size_t)top * a.nloc + loc) * 48) + k);
+                uint32_t *d = s_acc + 4 * (k & 1) * pitch + slot * 3 + (k >> 1);
+                d[0] = (v.x ^ 0x80008000u) - kB2;
+                d[pitch] = (v.y ^ 0x80008000u) - kB2;
+                d[2 * pitch] = (v.z ^ 0x80008000u) - kB2;
+                d[3 * pitch] = (v.w ^ 0x80008000u) - kB2;
+            }
+            // stored ancestor blocks of these requests, compacted
+            const uint32_t ntask = ns * 3 * nl;
+            uint32_t cnt = 0;
+            for (uint32_t t0 = 0; t0 < ntask; t0 += 32) {
+                const uint32_t t = t0 + lane;
+                uint32_t code = 0;
+                bool pres = false;
+                if (t < ntask) {
+                    const uint32_t slot = (t * inv3) >> 16, rem = t - slot * 3 * nl;
+                    const uint32_t c = (rem * inv1) >> 16, l = a.level + (rem - c * nl);
+                    const uint32_t node = ancestor(s_view[slot], l);
+                    const uint32_t wi = c * a.MW + (node >> 5), bit = node & 31u;
+                    const uint32_t word = s_mask[wi];
+                    pres = (word >> bit) & 1u;
+                    code = (s_mpre[wi] + __popc(word & ((1u << bit) - 1u))) | (c << 16) | (slot << 18);
                 }
-                const uint32_t pay0 = hdr0 + kHdrBits * total;
-                uint32_t run = 0;
-                for (uint32_t h0 = 0; h0 < total; h0 += 32) {
-                    const uint32_t hi = h0 + lane;
-                    const uint32_t len = hi < total ? mode_bits(s_modes[get_bits(rc, hdr0 + kHdrBits * hi, 5)]) : 0u;
-                    const uint32_t incl = scan_incl(len, lane);
-                    if (hi < total)
-                        s_off[c * a.pmax + hi] = pay0 + run + incl - len;
-                    run += __shfl_sync(kFull, incl, 31);
+                const uint32_t bal = __ballot_sync(kFull, pres);
+                if (pres)
+                    s_list[cnt + __popc(bal & ((1u << lane) - 1u))] = code;
+                cnt += __popc(bal);
+            }
+            __syncwarp();
+            // BISEDecode + CombineBlocks, one thread per stored block
+            for (uint32_t i = lane; i < cnt; i += 32) {
+                const uint32_t code = s_list[i];
+                const uint32_t at = code & 0xFFFFu, c = (code >> 16) & 3u, slot = code >> 18;   // at: among the three records' blocks
+                const uint32_t rank = at - (c == 0 ? 0u : (c == 1 ? p1 : p2));
+                const uint32_t *rc = rec_of(c);
+                const uint32_t hdr = get_bits(rc, hdr0 + kHdrBits * rank, kHdrBits), pos = s_off[at];
+#ifdef RLFC_DEBUG
+                {
+                    const uint32_t mode = hdr & 31u;
+                    const uint32_t rec_words = c == 0 ? d1 : (c == 1 ? d2 - d1 : span - d2);
+                    const uint32_t P = c == 0 ? p1 : (c == 1 ? p2 - p1 : total - p2);
+                    if (!RLFC_DBG_BLOCK_OK(a.dbg, mode, hdr0 + kHdrBits * (rank + 1), hdr0 + kHdrBits * P, pos,
+                                           mode < (uint32_t)kNumModes ? mode_bits(s_mode[mode]) : 0u, 32u * rec_words))
+                        continue;
+                }
+#endif
+                uint32_t v[8];
+                decode_block_pairs(rc, pos, hdr, a.q, s_mode, s_dig, v);
+                uint32_t *dst = s_acc + slot * 3 + c;
+#pragma unroll
+                for (int j = 0; j < 8; j++)
+                    atomicAdd(dst + j * pitch, v[j] - kB2);
+            }
+            __syncwarp();
+            // a lane per block row
+            for (uint32_t t0 = 0; t0 < 4 * ns; t0 += 32) {
+                const uint32_t t = t0 + lane, slot = min(t >> 2, ns - 1), rr = t & 3u;
+                const uint32_t *p = s_acc + 2 * rr * pitch + slot * 3;
+                uint32_t w[4];
+                row_to_rgb<false>(make_uint2(p[0], p[pitch]), make_uint2(p[1], p[pitch + 1]), make_uint2(p[2], p[pitch + 2]), w);
+                uint8_t *o = a.out + (size_t)s_req[slot] * 48;
+                if (a.aligned == 16) {
+                    // rows of 12 bytes to three 16-byte pieces: row rr gives its
+                    // piece rr the words it holds of it, row rr + 1 the rest
+                    const uint32_t n0 = __shfl_down_sync(kFull, w[0], 1), n1 = __shfl_down_sync(kFull, w[1], 1),
+                                   n2 = __shfl_down_sync(kFull, w[2], 1);
+                    const uint4 v = rr == 0 ? make_uint4(w[0], w[1], w[2], n0)
+                                            : (rr == 1 ? make_uint4(w[1], w[2], n0, n1) : make_uint4(w[2], n0, n1, n2));
+                    if (t < 4 * ns && rr < 3)
+                        reinterpret_cast<uint4 *>(o)[rr] = v;
+                } else if (t < 4 * ns) {
+                    if (a.aligned == 4) {
+#pragma unroll
+                        for (int k = 0; k < 3; k++)
+                            reinterpret_cast<uint32_t *>(o)[3 * rr + k] = w[k];
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 12; k++)
+                            o[12 * rr + k] = (uint8_t)(w[k >> 2] >> (8 * (k & 3)));
+                    }
                 }
             }
             __syncwarp();
-            for (uint32_t j0 = r0; j0 < r1; j0 += kSlots) {
-                const uint32_t ns = min(kSlots, r1 - j0);
-                if ((uint32_t)lane < ns) {
-                    s_req[lane] = a.sorted[j0 + lane];
-                    s_view[lane] = a.sorted_view[j0 + lane];
-                }
-                __syncwarp();
-                // ReadBlock(RKV^n, BlkIdx): the accumulators start at the top RKV
-                // (96 bytes per slot, as six 16-byte loads)
-                for (uint32_t i = lane; i < ns * 6; i += 32) {
-                    const uint32_t slot = i / 6, k = i - slot * 6;
-                    const uint32_t top = view_anc[s_view[slot] * kMaxLevels + a.L - 1];
-                    const uint4 v = reinterpret_cast<const uint4 *>(a.top + ((size_t)top * a.nloc + loc) * 48)[k];
-                    int32_t *d = s_acc + slot * 48 + k * 8;
-                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        d[2 * e] = (int32_t)(int16_t)(w[e] & 0xFFFFu);
-                        d[2 * e + 1] = (int32_t)w[e] >> 16;
-                    }
-                }
-                // stored ancestor blocks of these requests, compacted
-                const uint32_t ntask = ns * 3 * nl;
-                uint32_t cnt = 0;
-                for (uint32_t t0 = 0; t0 < ntask; t0 += 32) {
-                    const uint32_t t = t0 + lane;
-                    uint32_t code = 0;
-                    bool pres = false;
-                    if (t < ntask) {
-                        const uint32_t slot = t / (3 * nl), rem = t - slot * 3 * nl;
-                        const uint32_t c = rem / nl, l = a.level + (rem - c * nl);
-                        const uint32_t node = view_anc[s_view[slot] * kMaxLevels + l];
-                        const uint32_t wi = node >> 5, bit = node & 31u;
-                        const uint32_t word = s_mask[c * a.MW + wi];
-                        pres = (word >> bit) & 1u;
-                        const uint32_t rank = s_mpre[c * a.MW + wi] + __popc(word & ((1u << bit) - 1u));
-                        code = rank | (c << 16) | (slot << 18);
-                    }
-                    const uint32_t bal = __ballot_sync(kFull, pres);
-                    if (pres)
-                        s_list[cnt + __popc(bal & ((1u << lane) - 1u))] = code;
-                    cnt += __popc(bal);
-                }
-                __syncwarp();
-                // BISEDecode + CombineBlocks, one thread per stored block
-                for (uint32_t i = lane; i < cnt; i += 32) {
-                    const uint32_t code = s_list[i];
-                    const uint32_t rank = code & 0xFFFFu, c = (code >> 16) & 3u, slot = code >> 18;
-                    const uint32_t *rc = base + (c == 0 ? 0u : (c == 1 ? d1 : d2));
-                    const BlockHeader h = unpack_header(get_bits(rc, hdr0 + kHdrBits * rank, kHdrBits));
-#ifdef RLFC_DEBUG
-                    {
-                        const uint32_t rec_words = c == 0 ? d1 : (c == 1 ? d2 - d1 : span - d2);
-                        const uint32_t P = s_mpre[c * a.MW + a.MW - 1] + __popc(s_mask[c * a.MW + a.MW - 1]);
-                        if (!RLFC_DBG_BLOCK_OK(a.dbg, h.mode, hdr0 + kHdrBits * (rank + 1), hdr0 + kHdrBits * P,
-                                               s_off[c * a.pmax + rank],
-                                               h.mode < (uint32_t)kNumModes ? mode_bits(s_modes[h.mode]) : 0u,
-                                               32u * rec_words))
-                            continue;
-                    }
-#endif
-                    int32_t u[kVals];
-                    bise_decode16(rc, s_off[c * a.pmax + rank], s_modes[h.mode], u);
-                    const int32_t scale = 1 << (a.q + h.shift);
-                    int32_t *dst = s_acc + slot * 48 + c * 16;
-#pragma unroll
-                    for (int v = 0; v < kVals; v++)
-                        atomicAdd(&dst[v], (h.min + u[v]) * scale);
-                }
-                __syncwarp();
-                for (uint32_t i = lane; i < ns * 16; i += 32) {
-                    const uint32_t slot = i >> 4, k = i & 15u;
-                    const int32_t *acc = s_acc + slot * 48;
-                    s_rgb[i] = ycocg_to_rgb24(acc[k], acc[16 + k], acc[32 + k]);
-                }
-                __syncwarp();
-                if (a.aligned) {
-                    // 48 bytes as 12 words; word w starts at byte (4w) % 3 of
-                    // pixel (4w) / 3 and ends inside the next pixel
-                    for (uint32_t i = lane; i < ns * 12; i += 32) {
-                        const uint32_t slot = i / 12, wd = i - slot * 12;
-                        const uint32_t p0 = (4 * wd) / 3;
-                        const uint32_t lo = s_rgb[slot * 16 + p0], hi = s_rgb[slot * 16 + p0 + 1];
-                        const uint32_t sh = (4 * wd) % 3;   // first byte of the word inside pixel p0
-                        reinterpret_cast<uint32_t *>(a.out + (size_t)s_req[slot] * 48)[wd] =
-                            __byte_perm(lo, hi, sh == 0 ? 0x4210u : (sh == 1 ? 0x5421u : 0x6542u));
-                    }
-                } else {
-                    for (uint32_t i = lane; i < ns * 48; i += 32) {
-                        const uint32_t slot = i / 48, byte = i - slot * 48;
-                        a.out[(size_t)s_req[slot] * 48 + byte] = (uint8_t)(s_rgb[slot * 16 + byte / 3] >> (8 * (byte % 3)));
-                    }
-                }
-                __syncwarp();
-            }
         }
     };
 
@@ -439,12 +466,12 @@ struct rlfc_batch {
     const rlfc_stream *s = nullptr;
     int device = 0;
     size_t max_n = 0;
-    uint32_t nloc = 0, pmax = 1, stage_words = 0, smem_optin = 0, sms = 0;
+    uint32_t nloc = 0, pmax = 1, stage_words = 0, smem_optin = 0, smem_dyn = 0, sms = 0;   // smem_dyn: what the kernel has besides its static part
     uint32_t *d_cnt = nullptr;      // nloc + 2 words, then one per scan chunk
     uint32_t *d_rank = nullptr;     // max_n
-    uint32_t *d_sorted = nullptr;   // max_n
-    uint32_t *d_sorted_view = nullptr;   // max_n
-    uint32_t anc_words = 0;         // ancestor-table words cached per CTA (0 = none)
+    uint2 *d_sorted = nullptr;      // max_n
+    uint32_t anc_views = 0;         // views whose ancestors are cached per CTA (0 = none)
+    uint32_t off_bytes = 4;         // bytes of a payload offset: 2 while every record is shorter than 2^16 bits
     rlfc_batch_config cfg{8, 1, 0, 1};
     cudaStream_t cap = nullptr;     // private stream, only ever capturing
     cudaGraphExec_t exec = nullptr;
@@ -463,13 +490,30 @@ struct rlfc_batch {
 namespace rlfc {
 namespace {
 
-uint32_t smem_bytes(const rlfc_batch *b, const rlfc_batch_config &c)
+uint32_t warp_words(const rlfc_batch *b, const rlfc_batch_config &c, uint32_t slots)
 {
-    return c.warps_per_cta * 4u * warp_words_for(b->s->MW, b->pmax, b->s->tab.L, c.stage, b->stage_words) +
-           4u * b->anc_words;
+    return warp_words_for(b->s->MW, b->pmax, b->s->tab.L, c.stage, b->stage_words, b->off_bytes, slots);
+}
+uint32_t smem_bytes(const rlfc_batch *b, const rlfc_batch_config &c, uint32_t slots)
+{
+    return c.warps_per_cta * 4u * warp_words(b, c, slots) + 2u * kMaxLevels * b->anc_views;
+}
+uint32_t slots_for(const rlfc_batch *b, const rlfc_batch_config &c)
+{
+    return smem_bytes(b, c, kSlots) <= b->smem_dyn ? kSlots : kSlotsTight;
 }
 
-bool fits(const rlfc_batch *b, const rlfc_batch_config &c) { return smem_bytes(b, c) <= b->smem_optin; }
+bool fits(const rlfc_batch *b, const rlfc_batch_config &c)
+{
+    return c.warps_per_cta * 4u * warp_words_limit(b->s->MW, b->pmax, b->s->tab.L, c.stage, b->stage_words) +
+               4u * kMaxLevels * b->anc_views <= b->smem_optin - kStaticLimit;
+}
+
+using BinnedKernel = void (*)(const DecArgs);
+BinnedKernel binned_kernel(uint32_t off_bytes)
+{
+    return off_bytes == 2 ? decode_binned_kernel<uint16_t> : decode_binned_kernel<uint32_t>;
+}
 
 int enqueue(rlfc_batch *b, const rlfc_batch_config &cfg, const uint32_t *view, const uint32_t *loc, uint32_t n,
             uint32_t level, uint8_t *out, uint8_t *status, cudaStream_t st)
@@ -486,7 +530,6 @@ int enqueue(rlfc_batch *b, const rlfc_batch_config &cfg, const uint32_t *view, c
     ba.cnt = b->d_cnt;
     ba.rank = b->d_rank;
     ba.sorted = b->d_sorted;
-    ba.sorted_view = b->d_sorted_view;
     ba.n = n;
     ba.n_views = s->tab.n_views;
     ba.nloc = b->nloc;
@@ -505,11 +548,10 @@ int enqueue(rlfc_batch *b, const rlfc_batch_config &cfg, const uint32_t *view, c
     da.offsets = s->d_offsets;
     da.top = s->d_top;
     da.view_anc = s->d_view_anc;
-    da.req_view = view;
     da.start = b->d_cnt;
     da.sorted = b->d_sorted;
-    da.sorted_view = b->d_sorted_view;
-    da.anc_words = b->anc_words;
+    da.anc_views = b->anc_views;
+    da.slots = slots_for(b, cfg);
     da.out = out;
     da.queue = b->d_cnt + b->nloc + 1;
     da.nloc = b->nloc;
@@ -521,15 +563,16 @@ int enqueue(rlfc_batch *b, const rlfc_batch_config &cfg, const uint32_t *view, c
     da.locs_per_pop = cfg.locs_per_pop;
     da.stage = cfg.stage;
     da.stage_words = b->stage_words;
-    da.warp_words = warp_words_for(s->MW, b->pmax, s->tab.L, cfg.stage, b->stage_words);
-    da.aligned = ba.aligned;
-    const uint32_t threads = cfg.warps_per_cta * 32, smem = smem_bytes(b, cfg);
+    da.warp_words = warp_words(b, cfg, da.slots);
+    da.aligned = ((uintptr_t)out & 15u) == 0 ? 16u : (ba.aligned ? 4u : 1u);
+    const uint32_t threads = cfg.warps_per_cta * 32, smem = smem_bytes(b, cfg, da.slots);
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_binned_kernel, (int)threads, smem);
+    const BinnedKernel kern = binned_kernel(b->off_bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)threads, smem);
     if (e != cudaSuccess)
         return cuda_fail(e, "batch occupancy");
     const uint32_t grid = b->sms * (uint32_t)std::max(per_sm, 1);
-    { TraceScope trace_("decode_binned_kernel", st); decode_binned_kernel<<<grid, threads, smem, st>>>(da); }
+    { TraceScope trace_("decode_binned_kernel", st); kern<<<grid, threads, smem, st>>>(da); }
     e = cudaGetLastError();
     if (e != cudaSuccess)
         return cuda_fail(e, "batch decode launch");
@@ -591,7 +634,8 @@ RLFC_API int rlfc_batch_create(const rlfc_stream *s, size_t max_requests, rlfc_b
     b->pmax = std::max<uint32_t>(s->max_present, 1u);
     b->stage_words = std::min<uint32_t>(3u * s->max_record_words, kStageCap);
     // the ancestor table is cached per CTA up to 1024 views
-    b->anc_words = s->tab.n_views <= 1024u ? s->tab.n_views * (uint32_t)kMaxLevels : 0u;
+    b->anc_views = s->tab.n_views <= 1024u ? s->tab.n_views : 0u;
+    b->off_bytes = s->max_record_words < 2048u ? 2u : 4u;
     int v = 0;
     cudaError_t e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device);
     b->smem_optin = e == cudaSuccess ? (uint32_t)v : 48u * 1024u;
@@ -600,12 +644,12 @@ RLFC_API int rlfc_batch_create(const rlfc_stream *s, size_t max_requests, rlfc_b
     b->sms = (uint32_t)v;
     cudaFuncAttributes fa{};
     if (e == cudaSuccess)
-        e = cudaFuncGetAttributes(&fa, decode_binned_kernel);
+        e = cudaFuncGetAttributes(&fa, binned_kernel(b->off_bytes));
     if (e == cudaSuccess) {
         // the opt-in limit covers static and dynamic shared memory together
-        b->smem_optin -= std::min<uint32_t>(b->smem_optin, (uint32_t)fa.sharedSizeBytes);
-        e = cudaFuncSetAttribute(decode_binned_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)b->smem_optin);
+        b->smem_dyn = b->smem_optin - std::min<uint32_t>(b->smem_optin, (uint32_t)fa.sharedSizeBytes);
+        e = cudaFuncSetAttribute(binned_kernel(b->off_bytes), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)b->smem_dyn);
     }
     if (e != cudaSuccess) {
         delete b;
@@ -622,8 +666,7 @@ RLFC_API int rlfc_batch_create(const rlfc_stream *s, size_t max_requests, rlfc_b
     const size_t chunks = (b->nloc + kScanChunk - 1) / kScanChunk;
     if ((e = cudaMalloc(&b->d_cnt, (size_t)(b->nloc + 2 + chunks) * 4)) != cudaSuccess ||
         (e = cudaMalloc(&b->d_rank, b->max_n * 4)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_sorted, b->max_n * 4)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_sorted_view, b->max_n * 4)) != cudaSuccess ||
+        (e = cudaMalloc(&b->d_sorted, b->max_n * 8)) != cudaSuccess ||
         (e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking)) != cudaSuccess) {
         const int rc = e == cudaErrorMemoryAllocation ? RLFC_E_OOM : RLFC_E_CUDA;
         cuda_fail(e, "rlfc_batch_create");
@@ -780,7 +823,6 @@ RLFC_API void rlfc_batch_free(rlfc_batch *b)
     cudaFree(b->d_cnt);
     cudaFree(b->d_rank);
     cudaFree(b->d_sorted);
-    cudaFree(b->d_sorted_view);
     delete b;
 }
 
