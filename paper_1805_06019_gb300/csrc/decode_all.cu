@@ -58,14 +58,15 @@ namespace {
 
 constexpr int kNL = (int)kDecodeStrip;          // block locations per CTA
 constexpr int kRecs = 3 * kNL;
-constexpr int kThreads = 384;                    // twelve warps: eight parse the strip's locations, all twelve take view units
-constexpr int kWarps = kThreads / 32;
+constexpr int kWarps = 12;                       // warps per CTA at most
+constexpr int kThreads = 32 * kWarps;
 constexpr int kUnit = 8;                         // BFS positions per unit of view work (a quarter mask word)
 constexpr int kWSlots = 32;                      // decode slots per warp
 constexpr int kZeroSlot = kWSlots;               // a slot of zero residuals, for channels without a stored block
 constexpr int kWItems = kNL * kUnit;             // items per warp at most (every block of a unit)
-constexpr uint32_t kSmemBudget = 200 * 1024;
-constexpr size_t kCtaSmemTarget = 111 * 1024;    // two CTAs per SM (with the static arrays and the 1 KB each CTA reserves): staging fills up to this
+constexpr uint32_t kSmemBudget = 200 * 1024 + 16 * 2 * kWarps + 4 * kWItems * kWarps;   // larger trees are refused
+constexpr size_t kSmSmem = 228 * 1024;           // shared memory of an SM, and what a CTA takes of it besides its dynamic part
+constexpr size_t kCtaOwn = 1024 + 1536;
 constexpr uint32_t kNodeSmemMax = 4096;          // node tables up to this size are cached per CTA
 
 static_assert(kNL == 8, "the location and group splits below assume eight locations per strip");
@@ -73,6 +74,23 @@ static_assert(3 * kNL <= 32 && (kNL & (kNL - 1)) == 0, "the strip's records fit 
 static_assert(kUnit == 8, "a unit is a quarter of a 32-bit mask word");
 static_assert(kNL == 8 && kUnit * 4 == 32, "the list builder's lanes are (view of the unit, quarter of the strip)");
 static_assert(kWSlots >= 6, "one lane's slots (two locations, three channels) must fit a run");
+
+// Shared-memory layout of a CTA: 32-bit word offsets, computed once on the host.
+struct Layout {
+    uint32_t slots;   // [warp][kWSlots + 1][8]  decoded blocks, biased pairs; slot kZeroSlot is zero
+    uint32_t top;     // [n_top][kNL][24]  biased pairs
+    uint32_t inter;   // [n_int][kNL][24]  internal reconstructions, biased pairs
+    uint32_t mask;    // [kRecs][MW]
+    uint32_t mpre;    // [kRecs][MW]  stored blocks in front of each mask word
+    uint32_t need;    // [MW]  views to decode (bit per BFS position)
+    uint32_t node;    // [S]  node table (when cached)
+    uint32_t sent;    // [warp][kWSlots]  record | rank << 8
+    uint32_t items;   // [warp][kWItems] uint2: parent's block and the item's place in the buffer; its channels' slots
+    uint32_t obuf;    // [warp][kUnit][4][kNL * 4 * bytes per pixel]  the unit's output rows
+    uint32_t prgb;    // [n_par][4][kNL][row_words]  parent rows converted to RGB
+    uint32_t off;     // [pmax]  payload bit offset of each stored block (OffT), record after record
+    uint32_t stage;   // [stage_words]  the strip's records, from a 16-byte boundary
+};
 
 struct Args {
     const uint32_t *records;
@@ -95,6 +113,8 @@ struct Args {
     uint32_t lvl_begin[kMaxLevels];  // first BFS position of each internal level, top level first; [L-2] = n_int
     uint32_t *dbg;           // debug builds: the stream's flag word
     uint32_t n_out;          // output views (or slots of the packed instantiation)
+    Layout at;               // where the shared-memory arrays start
+    uint32_t warps;          // warps per CTA
     uint32_t ahead;          // CTAs resident at once: the strip this many ahead is prefetched into L2
 };
 
@@ -106,60 +126,32 @@ __host__ __device__ constexpr uint32_t row_words() { return kPacked ? 4u : 3u; }
 template <bool kPacked>
 __host__ __device__ constexpr uint32_t obuf_words() { return kUnit * 4 * kNL * row_words<kPacked>() / 4 + 2; }
 
-struct Smem {
-    uint32_t *slots;   // [warp][kWSlots + 1][8]  decoded blocks, biased pairs; slot kZeroSlot is zero
-    uint32_t *top;     // [n_top][kNL][24]  biased pairs
-    uint32_t *inter;   // [n_int][kNL][24]  internal reconstructions, biased pairs
-    uint32_t *mask;    // [kRecs][MW]
-    uint32_t *mpre;    // [kRecs][MW]  stored blocks in front of each mask word
-    uint32_t *need;    // [MW]  views to decode (bit per BFS position)
-    uint32_t *node;    // [S]  node table (when cached)
-    uint32_t *sent;    // [warp][kWSlots]  record | rank << 8
-    uint32_t *items;   // [warp][kWItems]  p | l << 14 | stored channels << 18 | first slot << 21
-    uint32_t *obuf;    // [warp][kUnit][4][kNL * 4 * bytes per pixel]  the unit's output rows
-    uint32_t *prgb;    // [n_par][4][kNL][row_words]  parent rows converted to RGB
-    void *off;         // [pmax]  payload bit offset of each stored block (OffT), record after record
-    uint32_t *stage;   // [stage_words]  the strip's records, from a 16-byte boundary
-};
+extern __shared__ __align__(16) uint32_t g_smem[];
 
-extern __shared__ __align__(16) unsigned char g_smem[];
-
-__host__ __device__ inline size_t r16(size_t b) { return (b + 15) & ~size_t(15); }
-
-// Shared-memory layout; the same function sizes it on the host (base null).
+// Fills the layout; returns its size in bytes.
 template <bool kPacked>
-__host__ __device__ inline size_t layout(unsigned char *base, const Args &a, size_t off_size, Smem *m)
+size_t layout(Args &a, size_t off_size)
 {
     size_t at = 0;
     auto take = [&](size_t bytes) {
-        unsigned char *p = base ? base + at : nullptr;
-        at += r16(bytes);
-        return p;
+        const size_t p = at;
+        at += (bytes + 15) & ~size_t(15);
+        return (uint32_t)(p / 4);
     };
-    Smem s;
-    s.slots = reinterpret_cast<uint32_t *>(take(32ull * (kWSlots + 1) * kWarps));
-    s.top = reinterpret_cast<uint32_t *>(take(96ull * a.n_top * kNL));
-    s.inter = reinterpret_cast<uint32_t *>(take(96ull * a.n_int * kNL));
-    s.mask = reinterpret_cast<uint32_t *>(take(4ull * kRecs * a.MW));
-    s.mpre = reinterpret_cast<uint32_t *>(take(4ull * kRecs * a.MW));
-    s.need = reinterpret_cast<uint32_t *>(take(4ull * a.MW));
-    s.node = reinterpret_cast<uint32_t *>(take(a.node_smem ? 4ull * a.S : 0));
-    s.sent = reinterpret_cast<uint32_t *>(take(4ull * kWSlots * kWarps));
-    s.items = reinterpret_cast<uint32_t *>(take(4ull * kWItems * kWarps));
-    s.obuf = reinterpret_cast<uint32_t *>(take(16ull * obuf_words<kPacked>() * kWarps));
-    s.prgb = reinterpret_cast<uint32_t *>(take(16ull * row_words<kPacked>() * a.n_par * kNL));
-    s.off = take(off_size * a.pmax);
-    s.stage = reinterpret_cast<uint32_t *>(take(4ull * a.stage_words));
-    if (m)
-        *m = s;
+    a.at.slots = take(32ull * (kWSlots + 1) * a.warps);
+    a.at.top = take(96ull * a.n_top * kNL);
+    a.at.inter = take(96ull * a.n_int * kNL);
+    a.at.mask = take(4ull * kRecs * a.MW);
+    a.at.mpre = take(4ull * kRecs * a.MW);
+    a.at.need = take(4ull * a.MW);
+    a.at.node = take(a.node_smem ? 4ull * a.S : 0);
+    a.at.sent = take(4ull * kWSlots * a.warps);
+    a.at.items = take(8ull * kWItems * a.warps);
+    a.at.obuf = take(16ull * obuf_words<kPacked>() * a.warps);
+    a.at.prgb = take(16ull * row_words<kPacked>() * a.n_par * kNL);
+    a.at.off = take(off_size * a.pmax);
+    a.at.stage = take(4ull * a.stage_words);
     return at;
-}
-
-// Address of pixel (x, y) of output view slot ov.
-template <bool kPacked>
-__device__ __forceinline__ uint8_t *out_px(const Args &a, uint32_t ov, uint32_t y, uint32_t x)
-{
-    return a.out + (((size_t)ov * a.H + y) * a.pitch + x) * (kPacked ? 4u : 3u);
 }
 
 template <bool kPacked, typename OffT>
@@ -175,20 +167,35 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
 #endif
     __shared__ uint32_t s_unit;   // next unit of view work
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t threads = blockDim.x, warps = a.warps;
     const uint32_t bx0 = blockIdx.x * kNL, by = blockIdx.y;
     const uint32_t nl = min((uint32_t)kNL, a.nlx - bx0);
     const uint32_t b0 = by * a.nlx + bx0;
-    Smem m;
-    layout<kPacked>(g_smem, a, sizeof(OffT), &m);
-    OffT *m_off = reinterpret_cast<OffT *>(m.off);
+    struct {
+        uint32_t *slots, *top, *inter, *mask, *mpre, *need, *node, *sent, *obuf, *prgb, *stage;
+        uint2 *items;
+    } m;
+    m.slots = g_smem + a.at.slots;
+    m.top = g_smem + a.at.top;
+    m.inter = g_smem + a.at.inter;
+    m.mask = g_smem + a.at.mask;
+    m.mpre = g_smem + a.at.mpre;
+    m.need = g_smem + a.at.need;
+    m.node = g_smem + a.at.node;
+    m.sent = g_smem + a.at.sent;
+    m.items = reinterpret_cast<uint2 *>(g_smem + a.at.items);
+    m.obuf = g_smem + a.at.obuf;
+    m.prgb = g_smem + a.at.prgb;
+    m.stage = g_smem + a.at.stage;
+    OffT *m_off = reinterpret_cast<OffT *>(g_smem + a.at.off);
     constexpr uint32_t RW = row_words<kPacked>();
     const uint32_t *nodes = a.node_smem ? m.node : a.node_info;
 
     // ---- set-up: tables, the strip's records and top-RKV blocks, zero reconstructions
     if (tid < 32)
         s_mode[tid] = g_tables.mode[tid];
-    if (tid < (256 + 128) / 2)
-        reinterpret_cast<uint32_t *>(s_dig)[tid] = reinterpret_cast<const uint32_t *>(g_tables.dig)[tid];
+    for (uint32_t i = tid; i < (256 + 128) / 2; i += threads)
+        reinterpret_cast<uint32_t *>(s_dig)[i] = reinterpret_cast<const uint32_t *>(g_tables.dig)[i];
     if (tid == 0)
         s_unit = 0;
     // the strip's records are contiguous in the stream: stage them (from a
@@ -200,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     if (staged) {
         const uint4 *src = reinterpret_cast<const uint4 *>(a.records + w_lo);
         uint4 *dst = reinterpret_cast<uint4 *>(m.stage);
-        for (uint32_t i = tid; i < n4; i += kThreads)
+        for (uint32_t i = tid; i < n4; i += threads)
             dst[i] = __ldg(src + i);
     }
     const uint32_t *rb = staged ? m.stage : a.records;   // records base: smem copy or stream
@@ -212,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     uint32_t pf_lo = 0, pf_hi = 0, pf_top = 0xFFFFFFFFu, pf_nl = 0;   // pf_top, pf_nl: the strip's first location and count
     {
         const uint32_t strip2 = blockIdx.y * gridDim.x + blockIdx.x + a.ahead;
-        if (warp == kWarps - 1 && a.ahead && strip2 < gridDim.x * gridDim.y) {
+        if (warp == (int)warps - 1 && a.ahead && strip2 < gridDim.x * gridDim.y) {
             const uint32_t bx2 = (strip2 % gridDim.x) * kNL, b02 = (strip2 / gridDim.x) * a.nlx + bx2;
             const uint32_t nl2 = min((uint32_t)kNL, a.nlx - bx2);
             pf_lo = __ldg(a.offsets + 3 * b02) & ~31u;
@@ -227,22 +234,22 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
 #endif
     {
         const uint32_t *tg = reinterpret_cast<const uint32_t *>(a.top);
-        for (uint32_t i = tid; i < a.n_top * kNL * 24; i += kThreads) {
+        for (uint32_t i = tid; i < a.n_top * kNL * 24; i += threads) {
             const uint32_t t = i / (kNL * 24), rest = i - t * (kNL * 24), loc = rest / 24, wi = rest - loc * 24;
             m.top[i] = loc < nl ? (__ldg(tg + ((size_t)t * a.nloc + b0 + loc) * 24 + wi) ^ 0x80008000u) - kB2 : kB2;
         }
     }
     uint32_t *wslots = m.slots + warp * (8 * (kWSlots + 1));   // this warp's slots
     uint32_t *wsent = m.sent + warp * kWSlots;
-    uint32_t *witems = m.items + warp * kWItems;
+    uint2 *witems = m.items + warp * kWItems;
     if (lane < 8)
         wslots[kZeroSlot * 8 + lane] = kB2;   // the warp's zero slot
     if (a.node_smem)
-        for (uint32_t i = tid; i < a.S; i += kThreads)
+        for (uint32_t i = tid; i < a.S; i += threads)
             m.node[i] = __ldg(a.node_info + i);
     __syncthreads();
     // the views to decode, one bit per BFS position (internal positions 0)
-    for (uint32_t w0 = warp * 32; w0 < a.MW * 32; w0 += kWarps * 32) {
+    for (uint32_t w0 = warp * 32; w0 < a.MW * 32; w0 += warps * 32) {
         const uint32_t p = w0 + lane;
         bool need = p >= a.n_int && p < a.S;
         if (need && kPacked && a.needed)
@@ -258,38 +265,59 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     // to RGB (a thread per (location, parent, block row))
     const uint32_t hdr0 = 32 * a.MW;
     // 1a. per record: mask words and the stored blocks in front of each
-    // (nothing stored past the end of the row)
-    for (uint32_t r = warp; r < (uint32_t)kRecs; r += kWarps) {
-        const bool live = r < 3 * nl;
-        uint32_t *mk = m.mask + r * a.MW;
-        uint32_t *mp = m.mpre + r * a.MW;
-        const uint32_t *rec = rb + s_roff[r];
-        uint32_t P = 0;
-        for (uint32_t w0 = 0; w0 < a.MW; w0 += 32) {
-            const uint32_t word = (live && w0 + lane < a.MW) ? rec[w0 + lane] : 0u;
-            const uint32_t cnt = (uint32_t)__popc(word);
-            const uint32_t incl = warp_inclusive_scan(cnt, lane);
-            if (w0 + lane < a.MW) {
-                mk[w0 + lane] = word;
-                mp[w0 + lane] = P + incl - cnt;
-            }
-            P += __shfl_sync(kFullMask, incl, 31);
+    // (nothing stored past the end of the row), and where the records' payload
+    // offsets start in m_off, record after record.  Masks of up to four words:
+    // one warp, a lane per record (a warp per record spends most of its lanes
+    // on nothing: 9 x 9 x 512^2, three words, 75 against 79 us); longer ones:
+    // a warp per record (eight words: 161 against 168 us).
+    const bool short_masks = a.MW <= 4;
+    uint32_t np_l = 0;
+    if (short_masks && warp == 0 && lane < kRecs) {
+        const bool live = (uint32_t)lane < 3 * nl;
+        const uint32_t *rec = rb + s_roff[lane];
+        for (uint32_t i = 0; i < a.MW; i++) {
+            const uint32_t word = live ? rec[i] : 0u;
+            m.mask[lane * a.MW + i] = word;
+            m.mpre[lane * a.MW + i] = np_l;
+            np_l += (uint32_t)__popc(word);
         }
-        if (lane == 0)
-            s_np[r] = P;
+        s_np[lane] = np_l;
+    }
+    if (!short_masks) {
+        for (uint32_t r = warp; r < (uint32_t)kRecs; r += warps) {
+            const bool live = r < 3 * nl;
+            uint32_t *mk = m.mask + r * a.MW;
+            uint32_t *mp = m.mpre + r * a.MW;
+            const uint32_t *rec = rb + s_roff[r];
+            uint32_t P = 0;
+            for (uint32_t w0 = 0; w0 < a.MW; w0 += 32) {
+                const uint32_t word = (live && w0 + lane < a.MW) ? rec[w0 + lane] : 0u;
+                const uint32_t cnt = (uint32_t)__popc(word);
+                const uint32_t incl = warp_inclusive_scan(cnt, lane);
+                if (w0 + lane < a.MW) {
+                    mk[w0 + lane] = word;
+                    mp[w0 + lane] = P + incl - cnt;
+                }
+                P += __shfl_sync(kFullMask, incl, 31);
+            }
+            if (lane == 0)
+                s_np[r] = P;
+        }
+        __syncthreads();
+        np_l = lane < kRecs ? s_np[lane] : 0u;
+    }
+    if (warp == 0) {
+        const uint32_t base = warp_inclusive_scan(np_l, lane) - np_l;
+        if (lane < kRecs)
+            s_obase[lane] = base;
     }
     __syncthreads();
-    // the strip's payload offsets go record after record into m_off
-    const uint32_t np_l = lane < kRecs ? s_np[lane] : 0u;
-    const uint32_t ob_l = warp_inclusive_scan(np_l, lane) - np_l;
-    if (warp == 0 && lane < kRecs)
-        s_obase[lane] = ob_l;
     // 1b. per record: payload offset of every stored block (closed-form
     // lengths of the 18-bit headers, warp scan)
-    for (uint32_t r = warp; r < 3 * nl; r += kWarps) {
+    for (uint32_t r = warp; r < 3 * nl; r += warps) {
         const uint32_t *rec = rb + s_roff[r];
         const uint32_t P = s_np[r];
-        OffT *o = m_off + __shfl_sync(kFullMask, ob_l, r);
+        OffT *o = m_off + s_obase[r];
         uint32_t run = hdr0 + kHdrBits * P;
         for (uint32_t h0 = 0; h0 < P; h0 += 32) {
             const uint32_t h = h0 + lane;
@@ -311,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     for (uint32_t lv = 0; lv + 2 < a.L; lv++) {
         const uint32_t g0 = a.lvl_begin[lv], g1 = a.lvl_begin[lv + 1];
         const uint32_t *src = lv == 0 ? m.top : m.inter;
-        for (uint32_t t = tid; t < (g1 - g0) * 3 * kNL; t += kThreads) {
+        for (uint32_t t = tid; t < (g1 - g0) * 3 * kNL; t += threads) {
             const uint32_t l = t & (kNL - 1), q = t / kNL;
             if (l >= nl)
                 continue;
@@ -351,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     // 3. the block rows of every parent of a view, as RGB
     {
         const uint32_t *src = a.L == 2 ? m.top : m.inter;
-        for (uint32_t t = tid; t < a.n_par * 4 * kNL; t += kThreads) {
+        for (uint32_t t = tid; t < a.n_par * 4 * kNL; t += threads) {
             const uint32_t l = t & (kNL - 1), q = t / kNL, n = q >> 2, rr = q & 3u;
             if (l >= nl)
                 continue;
@@ -366,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
         }
     }
     __syncthreads();
-    if (warp == kWarps - 1) {
+    if (warp == (int)warps - 1) {
         for (uint32_t i = pf_lo + 32u * lane; i < pf_hi; i += 32u * 32u)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(a.records + i)));
         // the strip's top-RKV blocks: 96 bytes per location, per top RKV
@@ -391,6 +419,11 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
     const bool whole = a.vec16 && bx0 * 4 + kNL * 4 <= a.pitch;
     // otherwise the strip row's bytes (the image may end inside the strip)
     const uint32_t piece = min(nl * 4u, a.W - bx0 * 4u) * BPP;
+    // this lane's piece of a view's strip: its 16-byte chunk, or, for the
+    // unaligned writer, its row
+    const size_t view_bytes = (size_t)a.pitch * a.H * BPP;
+    uint8_t *out_lane = a.out + ((size_t)(by * 4 + (whole ? (uint32_t)lane / CH : (uint32_t)lane >> 3)) * a.pitch + bx0 * 4) * BPP +
+                        (whole ? 16u * ((uint32_t)lane % CH) : 0u);
     for (;;) {
         uint32_t u = 0;
         if (lane == 0)
@@ -402,32 +435,37 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
         const uint32_t P0 = max(u * kUnit, a.n_int), P1 = min(u * kUnit + kUnit, a.S);
         const uint32_t lo = P0 - w * 32, hi = P1 - w * 32;
         const uint32_t sel = (hi >= 32 ? 0xFFFFFFFFu : ((1u << hi) - 1u)) & ~((1u << lo) - 1u) & m.need[w];
-        // per view of the unit (lane v < kUnit): its parent's rows and its
-        // output rows
-        uint32_t par_v = 0;
-        uint8_t *out_v = a.out;
+        // per view of the unit (lane v < kUnit): its parent's rows and blocks,
+        // and its output rows
+        uint32_t par_v = 0, ov_v = 0;
+        bool bad = false;
         if ((uint32_t)lane < (uint32_t)kUnit && ((sel >> (ub + lane)) & 1u)) {
             const uint32_t info = nodes[w * 32 + ub + lane];
-            par_v = (node_parent(info) - a.par_base) * 4 * CH;
-            const uint32_t ov = a.slot_of ? __ldg(a.slot_of + node_view(info)) : node_view(info);
-            out_v = RLFC_DBG_INDEX_OK(a.dbg, ov, a.n_out) ? out_px<kPacked>(a, ov, by * 4, bx0 * 4) : nullptr;
+            par_v = node_parent(info);
+            ov_v = a.slot_of ? __ldg(a.slot_of + node_view(info)) : node_view(info);
+            bad = !RLFC_DBG_INDEX_OK(a.dbg, ov_v, a.n_out);
         }
+        // the unit's views, and those of them that go out
+        const uint32_t selv = (sel >> ub) & 0xFFu, goes = selv & ~__ballot_sync(kFullMask, bad);
         // (a) the buffer starts as every view's parent rows (RGB), the exact
         // result for every block without a stored residual; lane = (row,
         // chunk of the view row)
-        const uint32_t f_rr = (uint32_t)lane / CH, f_c = (uint32_t)lane % CH;
-        const bool f_act = (uint32_t)lane < 4 * CH;
+        const uint32_t f_rr = (uint32_t)lane / CH;
+        const uint32_t fill = (uint32_t)lane < 4 * CH ? selv : 0u;
+        const uint4 *prgb4 = reinterpret_cast<const uint4 *>(m.prgb) + lane;
 #pragma unroll
         for (uint32_t vv = 0; vv < (uint32_t)kUnit; vv++) {
-            const uint32_t pv = __shfl_sync(kFullMask, par_v, vv);
-            if (((sel >> (ub + vv)) & 1u) && f_act)
-                wbuf[vv * 4 * CH + lane] = reinterpret_cast<const uint4 *>(m.prgb)[pv + lane];
+            const uint32_t pv = (__shfl_sync(kFullMask, par_v, vv) - a.par_base) * 4 * CH;
+            if (fill & (1u << vv))
+                wbuf[vv * 4 * CH + lane] = prgb4[pv];
         }
         // (b) items and slots.  Lane = (view ub + v, quarter qd of the strip):
         // the stored channels of its two locations 2qd, 2qd + 1
         const uint32_t v = (uint32_t)lane & 7u, qd = (uint32_t)lane >> 3, bit = ub + v;
         const uint32_t lt = (1u << bit) - 1u;   // positions in front of this view in mask word w
-        const bool vsel = (sel >> bit) & 1u;
+        const bool vsel = (selv >> v) & 1u;
+        // this lane's first block of its view's parent, and its place in the buffer
+        const uint32_t place = (__shfl_sync(kFullMask, par_v, v) * kNL + 2 * qd) * 24 | ((v * 4 * kNL + 2 * qd) * RW) << 16;
         uint32_t f[2][3];   // channel masks (word w) of the lane's locations
         uint32_t st = 0;    // stored channels of location 2qd + j at bits 3j .. 3j + 2
         uint32_t ni = 0, ns = 0;
@@ -462,7 +500,12 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
                 for (uint32_t j = 0; j < 2; j++) {
                     const uint32_t s3 = (st >> (3 * j)) & 7u, l = 2u * qd + j;
                     if (s3) {
-                        witems[item++] = (w * 32 + bit) | (l << 14) | (s3 << 18) | (slot << 21);
+                        // slots of the channels, times 32: the stored ones in
+                        // order, the zero slot for the others
+                        const uint32_t zy = (s3 & 1u) ? slot : (uint32_t)kZeroSlot;
+                        const uint32_t zo = (s3 & 2u) ? slot + (s3 & 1u) : (uint32_t)kZeroSlot;
+                        const uint32_t zg = (s3 & 4u) ? slot + __popc(s3 & 3u) : (uint32_t)kZeroSlot;
+                        witems[item++] = make_uint2(place + j * (24u | RW << 16), zy << 5 | zo << 13 | zg << 21);
 #pragma unroll
                         for (uint32_t c = 0; c < 3; c++)
                             if ((s3 >> c) & 1u) {
@@ -500,13 +543,11 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
             __syncwarp();
             // items: parent + residual -> RGB into the buffer, four lanes per item, one block row each
             for (uint32_t t = lane; t < 4 * n_items; t += 32) {
-                const uint32_t it = witems[t >> 2], rr = t & 3u;
-                const uint32_t p = it & 0x3FFFu, l = (it >> 14) & 15u, s3 = (it >> 18) & 7u, s0 = it >> 21;
-                const uint32_t *ps = par_slab + (node_parent(nodes[p]) * kNL + l) * 24 + 2 * rr;
-                // slot of each channel's residual, or the zero slot
-                const uint32_t *ry = wslots + 8 * ((s3 & 1u) ? s0 : (uint32_t)kZeroSlot) + 2 * rr;
-                const uint32_t *rco = wslots + 8 * ((s3 & 2u) ? s0 + (s3 & 1u) : (uint32_t)kZeroSlot) + 2 * rr;
-                const uint32_t *rcg = wslots + 8 * ((s3 & 4u) ? s0 + __popc(s3 & 3u) : (uint32_t)kZeroSlot) + 2 * rr;
+                const uint2 it = witems[t >> 2];
+                const uint32_t rr = t & 3u;
+                const uint32_t *ps = par_slab + (it.x & 0xFFFFu) + 2 * rr;
+                const unsigned char *rs = reinterpret_cast<const unsigned char *>(wslots) + 8 * rr;
+                const unsigned char *ry = rs + (it.y & 0x1FE0u), *rco = rs + ((it.y >> 8) & 0x1FE0u), *rcg = rs + ((it.y >> 16) & 0x1FE0u);
                 const uint2 py = *reinterpret_cast<const uint2 *>(ps);
                 const uint2 pco = *reinterpret_cast<const uint2 *>(ps + 8);
                 const uint2 pcg = *reinterpret_cast<const uint2 *>(ps + 16);
@@ -517,7 +558,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
                 row_to_rgb<kPacked>(make_uint2(py.x + vy.x - kB2, py.y + vy.y - kB2),
                                     make_uint2(pco.x + vco.x - kB2, pco.y + vco.y - kB2),
                                     make_uint2(pcg.x + vcg.x - kB2, pcg.y + vcg.y - kB2), wv);
-                uint32_t *d = reinterpret_cast<uint32_t *>(wbuf) + ((p - w * 32 - ub) * 4 + rr) * (kNL * RW) + l * RW;
+                uint32_t *d = reinterpret_cast<uint32_t *>(wbuf) + (it.x >> 16) + rr * (kNL * RW);
 #pragma unroll
                 for (uint32_t k = 0; k < RW; k++)
                     d[k] = wv[k];
@@ -526,25 +567,24 @@ __global__ void __launch_bounds__(kThreads, 2) decode_all_kernel(const Args a)
             L0 = L1;
         }
         // (c) write the unit's rows: consecutive lanes, consecutive chunks of one view row
-        const size_t row_bytes = (size_t)a.pitch * BPP;
         if (whole) {
+            const uint32_t put = f_rr < nrows && (uint32_t)lane < 4 * CH ? goes : 0u;
 #pragma unroll
             for (uint32_t vv = 0; vv < (uint32_t)kUnit; vv++) {
-                uint8_t *o = reinterpret_cast<uint8_t *>(
-                    __shfl_sync(kFullMask, reinterpret_cast<unsigned long long>(out_v), vv));
-                if (((sel >> (ub + vv)) & 1u) && f_act && f_rr < nrows && o)
-                    reinterpret_cast<uint4 *>(o + f_rr * row_bytes)[f_c] = wbuf[vv * 4 * CH + lane];
+                const uint32_t ov = __shfl_sync(kFullMask, ov_v, vv);
+                if (put & (1u << vv))
+                    *reinterpret_cast<uint4 *>(out_lane + ov * view_bytes) = wbuf[vv * 4 * CH + lane];
             }
         } else if (!kPacked) {
             // rows not 16-byte aligned, or the right edge of the image: lane =
             // (row, 16-byte chunk of the destination)
             const uint32_t rr = (uint32_t)lane >> 3, ch = (uint32_t)lane & 7u;
+            const uint32_t put = rr < nrows ? goes : 0u;
 #pragma unroll 2
             for (uint32_t vv = 0; vv < (uint32_t)kUnit; vv++) {
-                uint8_t *o = reinterpret_cast<uint8_t *>(
-                    __shfl_sync(kFullMask, reinterpret_cast<unsigned long long>(out_v), vv));
-                if (((sel >> (ub + vv)) & 1u) && rr < nrows && o)
-                    store_row_unaligned(o + rr * row_bytes, reinterpret_cast<const uint32_t *>(wbuf + (vv * 4 + rr) * CH),
+                const uint32_t ov = __shfl_sync(kFullMask, ov_v, vv);
+                if (put & (1u << vv))
+                    store_row_unaligned(out_lane + ov * view_bytes, reinterpret_cast<const uint32_t *>(wbuf + (vv * 4 + rr) * CH),
                                         piece, ch);
             }
         }
@@ -608,14 +648,29 @@ int launch_decode(const rlfc_stream *s, uint8_t *d_out, const uint8_t *needed, c
     // unless a record reaches 2^16 bits
     const bool off16 = (uint64_t)s->max_record_words * 32 < 65536;
     const size_t off_size = off16 ? 2 : 4;
-    // staging for the largest strip's records (16-byte boundary, decoder
-    // slack), within what keeps three CTAs per SM; strips whose records do
-    // not fit read them from the stream
-    a.stage_words = 0;
-    const size_t base = layout<kPacked>(nullptr, a, off_size, nullptr);
-    const size_t room = base < kCtaSmemTarget ? (kCtaSmemTarget - base) / 4 : 0;
-    a.stage_words = (uint32_t)std::min<size_t>((size_t)((s->max_strip_words + 8 + 3 + 3) & ~3u), room & ~size_t(3));
-    const size_t smem = layout<kPacked>(nullptr, a, off_size, nullptr);
+    // three CTAs of eight warps per SM where a strip's tables and the records
+    // of most strips fit a third of its shared memory, else two of twelve:
+    // set-up, parse and internal nodes wait on memory and barriers, and more
+    // CTAs overlap them with the view work of the others.  Measured, three
+    // against two: 9 x 9 x 512^2 75 / 83 us, 32 of its views packed 64 / 70,
+    // 5 x 5 x 64^2 16.8 / 17.4; 17 x 17 x 1024^2, whose records then read
+    // from the stream, 706 / 693.  Strips whose records do not fit what is
+    // left read them from the stream.
+    const uint32_t strips = (a.nlx + kNL - 1) / kNL * s->info.nloc_y;
+    const size_t longest = 4ull * ((s->max_strip_words + 8 + 3 + 3) & ~3u);
+    const size_t most = std::min<size_t>(longest, 4ull * (s->record_words / strips) * 3 / 2 + 64);
+    size_t base = 0, room = 0;
+    for (uint32_t ctas = 3; ctas >= 2; ctas--) {
+        a.warps = 24 / ctas;
+        a.stage_words = 0;
+        base = layout<kPacked>(a, off_size);
+        const size_t have = kSmSmem / ctas - kCtaOwn;
+        room = base < have ? (have - base) & ~size_t(15) : 0;
+        if (room >= most)
+            break;
+    }
+    a.stage_words = (uint32_t)(std::min(room, longest) / 4);
+    const size_t smem = layout<kPacked>(a, off_size);
     if (smem > kSmemBudget || a.S >= 16384) {
         set_error("tree too large for the decode-all kernel's shared memory");
         return RLFC_E_UNSUPPORTED;
@@ -628,10 +683,10 @@ int launch_decode(const rlfc_stream *s, uint8_t *d_out, const uint8_t *needed, c
     {
         int sms = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device) == cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) == cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)(32 * a.warps), smem) == cudaSuccess)
             a.ahead = (uint32_t)(std::max(sms, 0) * std::max(per_sm, 0));
     }
-    { rlfc::TraceScope trace_((kPacked ? "decode_all_kernel<packed>" : "decode_all_kernel"), st); kern<<<grid, kThreads, smem, st>>>(a); }
+    { rlfc::TraceScope trace_((kPacked ? "decode_all_kernel<packed>" : "decode_all_kernel"), st); kern<<<grid, 32 * a.warps, smem, st>>>(a); }
     e = cudaGetLastError();
     if (e != cudaSuccess)
         return cuda_fail(e, "decode_all launch");
