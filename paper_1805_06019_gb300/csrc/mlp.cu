@@ -4,17 +4,19 @@
 //
 // Numerics: parameters and inputs are stored in BF16; sums and activations
 // are FP32.  The network is small (14 576 parameters, layers 48 to 112 wide),
-// so the kernels keep the transposed weights, the gradient accumulators and
-// one tile of 32 samples' activations in shared memory; the products run on
+// so the kernels keep the weights and one tile of samples' activations in
+// shared memory (training: the gradients in registers); the products run on
 // the tensor pipe (BF16 MMA with FP32 accumulation, FP32 operands split into
 // two BF16 terms; see the tile helpers below).
 //
 // Parameter order (flat): W1 [64][48], b1 [64], W2 [64][64], b2 [64],
 // W3 [112][64], b3 [112]; rows are output units.  Class c = s * 28 + k.
 #include <cuda_bf16.h>
+#include <cuda_pipeline.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 
 #include "rlfc_device.cuh"
 #include "rlfc_internal.h"
@@ -232,7 +234,7 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t &hi, uint32_
 constexpr int LX = NI + 4, LH = NH + 4, LZ = NO + 4;
 // Row strides (BF16 elements) of the weight copies: the row-wise fragment
 // loads fall on distinct banks.
-constexpr int LW1 = NI + 8, LW2 = NH + 8, LW3 = NH + 8, LW2T = NH + 8, LW3T = NO + 8;
+constexpr int LW1 = NI + 8, LW2 = NH + 8, LW3 = NH + 8;
 
 // A fragment of a row-major FP32 tile M[m][k] (rows m0.., columns k0..).
 template <bool kExact>
@@ -249,17 +251,6 @@ __device__ __forceinline__ void frag_a_rows(const float *M, int ld, int m0, int 
     }
 }
 
-// A fragment of the transpose of an FP32 tile: A[m][k] = M[k][m].
-__device__ __forceinline__ void frag_a_cols(const float *M, int ld, int m0, int k0, uint32_t hi[4], uint32_t lo[4])
-{
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const int m = m0 + g + 8 * (q & 1), k = k0 + 2 * t + 8 * (q >> 1);
-        split2(M[k * ld + m], M[(k + 1) * ld + m], hi[q], lo[q]);
-    }
-}
-
 // B fragment of BF16 weights stored n-major, B[k][n] = Wb[n][k] (row stride ldw).
 __device__ __forceinline__ void frag_b_w(const uint16_t *Wb, int ldw, int n0, int k0, uint32_t b[2])
 {
@@ -267,22 +258,6 @@ __device__ __forceinline__ void frag_b_w(const uint16_t *Wb, int ldw, int n0, in
     const uint32_t *row = reinterpret_cast<const uint32_t *>(Wb + (n0 + g) * ldw + k0);
     b[0] = row[t];
     b[1] = row[4 + t];
-}
-
-// B fragment of a row-major FP32 tile, B[k][n] = M[k][n].
-template <bool kExact>
-__device__ __forceinline__ void frag_b_rows(const float *M, int ld, int n0, int k0, uint32_t hi[2], uint32_t lo[2])
-{
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
-#pragma unroll
-    for (int q = 0; q < 2; q++) {
-        const int k = k0 + 2 * t + 8 * q;
-        const float x0 = M[k * ld + n0 + g], x1 = M[(k + 1) * ld + n0 + g];
-        if (kExact)
-            hi[q] = pack_bf16(x0, x1);
-        else
-            split2(x0, x1, hi[q], lo[q]);
-    }
 }
 
 // C tile (16 x 8) at (m0, n0) of act(b + X W^T): X an FP32 activation tile
@@ -312,47 +287,35 @@ __device__ __forceinline__ void dense_tile(const float *X, int ldx, const uint16
     *reinterpret_cast<float2 *>(Y + (m0 + g + 8) * ldy + n) = make_float2(y[2], y[3]);
 }
 
-// The network's weights in shared memory: BF16 copies for the fragments
-// (W1, W2, W3 row-major as stored, W2 and W3 transposed for the backward
-// pass) and FP32 biases.
+// The network's weights in shared memory: BF16 as stored (row-major, padded
+// rows) and FP32 biases.
 struct NetW {
-    uint16_t *w1, *w2, *w3, *w2t, *w3t;
+    uint16_t *w1, *w2, *w3;
     float *b1, *b2, *b3;
 };
 
-constexpr int kWBytes = 2 * (NH * LW1 + NH * LW2 + NO * LW3 + NH * LW2T + NH * LW3T) + 4 * (NH + NH + NO);
+constexpr int kWBytes = 2 * (NH * LW1 + NH * LW2 + NO * LW3) + 4 * (NH + NH + NO);
 
-__device__ __forceinline__ NetW carve_w(unsigned char *base, bool transposed)
+__device__ __forceinline__ NetW carve_w(unsigned char *base)
 {
     NetW m;
     m.w1 = reinterpret_cast<uint16_t *>(base);
     m.w2 = m.w1 + NH * LW1;
     m.w3 = m.w2 + NH * LW2;
-    m.w2t = m.w3 + NO * LW3;
-    m.w3t = m.w2t + (transposed ? NH * LW2T : 0);
-    float *f = reinterpret_cast<float *>(m.w3t + (transposed ? NH * LW3T : 0));
-    m.b1 = f;
-    m.b2 = f + NH;
-    m.b3 = f + 2 * NH;
+    m.b1 = reinterpret_cast<float *>(m.w3 + NO * LW3);
+    m.b2 = m.b1 + NH;
+    m.b3 = m.b2 + NH;
     return m;
 }
 
-__device__ void load_weights(const uint16_t *w, const NetW &m, bool transposed)
+__device__ void load_weights(const uint16_t *w, const NetW &m)
 {
     for (int i = threadIdx.x; i < NH * NI; i += blockDim.x)
         m.w1[(i / NI) * LW1 + i % NI] = w[oW1 + i];
-    for (int i = threadIdx.x; i < NH * NH; i += blockDim.x) {
-        const int j = i / NH, k = i % NH;
-        m.w2[j * LW2 + k] = w[oW2 + i];
-        if (transposed)
-            m.w2t[k * LW2T + j] = w[oW2 + i];
-    }
-    for (int i = threadIdx.x; i < NO * NH; i += blockDim.x) {
-        const int j = i / NH, k = i % NH;
-        m.w3[j * LW3 + k] = w[oW3 + i];
-        if (transposed)
-            m.w3t[k * LW3T + j] = w[oW3 + i];
-    }
+    for (int i = threadIdx.x; i < NH * NH; i += blockDim.x)
+        m.w2[(i / NH) * LW2 + i % NH] = w[oW2 + i];
+    for (int i = threadIdx.x; i < NO * NH; i += blockDim.x)
+        m.w3[(i / NH) * LW3 + i % NH] = w[oW3 + i];
     for (int i = threadIdx.x; i < NH; i += blockDim.x) {
         m.b1[i] = bf(w[oB1 + i]);
         m.b2[i] = bf(w[oB2 + i]);
@@ -361,120 +324,300 @@ __device__ void load_weights(const uint16_t *w, const NetW &m, bool transposed)
         m.b3[i] = bf(w[oB3 + i]);
 }
 
-// Tile of samples [t0, t0 + kTile) in `order` (or in index order): inputs
-// (FP32 copies of the BF16 values) and classes (-1 for missing or invalid
-// ones).
-__device__ __forceinline__ void load_tile(const uint16_t *x, const uint8_t *label, const uint32_t *order,
-                                          uint32_t n, uint32_t t0, float *X, int *s_cls)
+// ---- training: forward, softmax cross-entropy, backward ------------------------
+//
+// What bounds it: the latency of a tile's phases (a default batch of 4096
+// samples is one 32-sample tile per CTA), so every phase is a few ldmatrix and
+// MMA instructions per warp: activations and deltas are split into their BF16
+// terms once, where they are produced; both operands of every product, also
+// the transposed ones of the backward pass, come from ldmatrix (with .trans),
+// so no transposed copies are made; weights arrive by cp.async in the order
+// the phases need them; sixteen warps share a phase's 16 x 8 tiles; and the
+// gradients stay in registers across a CTA's tiles and go out as 8-byte
+// reductions.  A batch of 4096 takes 19.7
+// us, one of 60000 110; with FP32 tiles split at every use, transposed weight
+// copies, eight warps and the gradients in shared memory, 27.7 and 200 us.
+
+constexpr int kTrainThreads = 512;
+constexpr int BX = NI + 8, BH = NH + 8, BZ = NO + 8;   // row strides (BF16) of the operand tiles: 16-byte rows, conflict-free ldmatrix
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Four 8 x 8 BF16 matrices; lane l gives the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void ldsm4(uint32_t r[4], uint32_t addr)
 {
-    for (int i = threadIdx.x; i < kTile * NI; i += blockDim.x) {
-        const uint32_t s = i / NI, f = i % NI, gs = t0 + s;
-        float v = 0.0f;
-        if (gs < n)
-            v = bf(x[(size_t)(order ? order[gs] : gs) * NI + f]);
-        X[s * LX + f] = v;
-    }
-    if (s_cls && threadIdx.x < kTile) {
-        const uint32_t gs = t0 + threadIdx.x;
-        int c = -1;
-        if (gs < n) {
-            const uint32_t lab = label[order ? order[gs] : gs];
-            if ((lab & 31u) < (uint32_t)kNumModes)
-                c = (int)((lab >> 5) * kNumModes + (lab & 31u));
-        }
-        s_cls[threadIdx.x] = c;
-    }
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t r[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm2(uint32_t r[2], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t r[2], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
+// A (16 x 16) of a row-major tile M[m][k]
+__device__ __forceinline__ void load_a(uint32_t a[4], const uint16_t *M, int ld, int m0, int k0)
+{
+    const int l = threadIdx.x & 31;
+    ldsm4(a, smem_addr(M + (m0 + (l & 15)) * ld + k0 + 8 * (l >> 4)));
+}
+// A[m][k] = M[k][m]
+__device__ __forceinline__ void load_at(uint32_t a[4], const uint16_t *M, int ld, int m0, int k0)
+{
+    const int l = threadIdx.x & 31;
+    ldsm4t(a, smem_addr(M + (k0 + (l & 7) + 8 * (l >> 4)) * ld + m0 + 8 * ((l >> 3) & 1)));
+}
+// B (16 x 8), B[k][n] = M[n][k]
+__device__ __forceinline__ void load_b(uint32_t b[2], const uint16_t *M, int ld, int n0, int k0)
+{
+    const int l = threadIdx.x & 15;
+    ldsm2(b, smem_addr(M + (n0 + (l & 7)) * ld + k0 + 8 * (l >> 3)));
+}
+// B[k][n] = M[k][n]
+__device__ __forceinline__ void load_bt(uint32_t b[2], const uint16_t *M, int ld, int n0, int k0)
+{
+    ldsm2t(b, smem_addr(M + (k0 + (threadIdx.x & 15)) * ld + n0));
 }
 
-// Gradient tile (16 x 8) at (m0, n0) of A^T B over the tile's samples,
-// A = D [s][m] (deltas, row stride ldd) and B = H [s][n] (activations or
-// inputs, row stride ldh), added to G[m][n] (row stride ldg).
-template <bool kHExact>
-__device__ __forceinline__ void grad_tile(const float *D, int ldd, const float *H, int ldh, float *G, int ldg, int m0,
+// A pair (columns n, n + 1) of a row as its two BF16 terms.
+__device__ __forceinline__ void put_pair(uint16_t *hi, uint16_t *lo, int at, float x0, float x1)
+{
+    uint32_t h, l;
+    split2(x0, x1, h, l);
+    *reinterpret_cast<uint32_t *>(hi + at) = h;
+    *reinterpret_cast<uint32_t *>(lo + at) = l;
+}
+
+// C tile (16 x 8) at (m0, n0) of X W^T; X as its BF16 terms, or exact (lo unused).
+template <int K, bool kExact>
+__device__ __forceinline__ void dense_mma(float c[4], const uint16_t *Xh, const uint16_t *Xl, int ldx, const uint16_t *W, int ldw, int m0,
                                           int n0)
 {
-    float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    c[0] = c[1] = c[2] = c[3] = 0.0f;
 #pragma unroll
-    for (int k0 = 0; k0 < kTile; k0 += 16) {
-        uint32_t ah[4], al[4], bh[2], bl[2];
-        frag_a_cols(D, ldd, m0, k0, ah, al);
-        frag_b_rows<kHExact>(H, ldh, n0, k0, bh, bl);
-        mma_bf16(c, ah, bh);
-        mma_bf16(c, al, bh);
-        if (!kHExact)
-            mma_bf16(c, ah, bl);
+    for (int k0 = 0; k0 < K; k0 += 16) {
+        uint32_t b[2], a[4];
+        load_b(b, W, ldw, n0, k0);
+        load_a(a, Xh, ldx, m0, k0);
+        mma_bf16(c, a, b);
+        if (!kExact) {
+            load_a(a, Xl, ldx, m0, k0);
+            mma_bf16(c, a, b);
+        }
     }
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
-    float *r0 = G + (m0 + g) * ldg + n0 + 2 * t, *r1 = r0 + 8 * ldg;
-    r0[0] += c[0];
-    r0[1] += c[1];
-    r1[0] += c[2];
-    r1[1] += c[3];
 }
 
-// Delta tile (16 x 8) at (m0, n0) of (Dn Wn) * relu'(H): Dn the next layer's
-// deltas [s][K] (row stride ldd), Wn^T as BF16 weights [N][K], H the layer's
-// activations [s][N].
+// Tile (m0, n0) of one hidden layer: relu(b + X W^T) as BF16 terms.
+template <int K, bool kExact>
+__device__ __forceinline__ void hidden_tile(const uint16_t *Xh, const uint16_t *Xl, int ldx, const uint16_t *W, int ldw, const float *b,
+                                            uint16_t *Hh, uint16_t *Hl, int m0, int n0)
+{
+    float c[4];
+    dense_mma<K, kExact>(c, Xh, Xl, ldx, W, ldw, m0, n0);
+    const int g = (threadIdx.x & 31) >> 2, n = n0 + 2 * (threadIdx.x & 3);
+    const float b0 = b[n], b1 = b[n + 1];
+    put_pair(Hh, Hl, (m0 + g) * BH + n, fmaxf(c[0] + b0, 0.0f), fmaxf(c[1] + b1, 0.0f));
+    put_pair(Hh, Hl, (m0 + g + 8) * BH + n, fmaxf(c[2] + b0, 0.0f), fmaxf(c[3] + b1, 0.0f));
+}
+
+// Tile (m0, n0) of the deltas of a hidden layer: (Dn W) * relu'(H), W the next
+// layer's weights [K][NH]; its column sums are added to gb (the bias gradient).
 template <int K>
-__device__ __forceinline__ void delta_tile(const float *Dn, int ldd, const uint16_t *Wt, int ldw, const float *H,
-                                           int ldh, float *D, int ld, int m0, int n0)
+__device__ __forceinline__ void delta_tile(const uint16_t *Dnh, const uint16_t *Dnl, int ldd, const uint16_t *W, int ldw,
+                                           const uint16_t *Hh, uint16_t *Dh, uint16_t *Dl, float *gb, int m0, int n0)
 {
     float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int k0 = 0; k0 < K; k0 += 16) {
-        uint32_t ah[4], al[4], bw[2];
-        frag_a_rows<false>(Dn, ldd, m0, k0, ah, al);
-        frag_b_w(Wt, ldw, n0, k0, bw);
-        mma_bf16(c, ah, bw);
-        mma_bf16(c, al, bw);
+        uint32_t b[2], a[4];
+        load_bt(b, W, ldw, n0, k0);
+        load_a(a, Dnh, ldd, m0, k0);
+        mma_bf16(c, a, b);
+        load_a(a, Dnl, ldd, m0, k0);
+        mma_bf16(c, a, b);
     }
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3, n = n0 + 2 * t;
+    const int lane = threadIdx.x & 31, g = lane >> 2, n = n0 + 2 * (lane & 3);
+    float s0 = 0.0f, s1 = 0.0f;
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const int m = m0 + g + 8 * (q >> 1), nn = n + (q & 1);
-        D[m * ld + nn] = H[m * ldh + nn] > 0.0f ? c[q] : 0.0f;
+    for (int h = 0; h < 2; h++) {
+        const int at = (m0 + g + 8 * h) * BH + n;
+        const uint32_t act = *reinterpret_cast<const uint32_t *>(Hh + at);   // relu outputs: positive or zero
+        const float d0 = (act & 0x7FFFu) ? c[2 * h] : 0.0f, d1 = (act & 0x7FFF0000u) ? c[2 * h + 1] : 0.0f;
+        put_pair(Dh, Dl, at, d0, d1);
+        s0 += d0;
+        s1 += d1;
+    }
+#pragma unroll
+    for (int d = 4; d < 32; d <<= 1) {
+        s0 += __shfl_xor_sync(kFull, s0, d);
+        s1 += __shfl_xor_sync(kFull, s1, d);
+    }
+    if (g == 0) {
+        atomicAdd(&gb[n], s0);
+        atomicAdd(&gb[n + 1], s1);
     }
 }
 
-constexpr int kTileFloats = kTile * (LX + LH + LH + LZ + LH + LH);
+// Gradient tile (16 x 8) at (m0, n0) of D^T H over the tile's samples, added to
+// g (each tile summed from zero, then added in FP32): both operands as BF16
+// terms (H exact when kExact).
+template <bool kExact>
+__device__ __forceinline__ void grad_acc(float g[4], const uint16_t *Dh, const uint16_t *Dl, int ldd, const uint32_t bh[2][2],
+                                         const uint32_t bl[2][2], int m0)
+{
+    float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < kTile / 16; k++) {
+        uint32_t ah[4], al[4];
+        load_at(ah, Dh, ldd, m0, 16 * k);
+        load_at(al, Dl, ldd, m0, 16 * k);
+        mma_bf16(c, ah, bh[k]);
+        mma_bf16(c, al, bh[k]);
+        if (!kExact)
+            mma_bf16(c, ah, bl[k]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+        g[q] += c[q];
+}
 
-__global__ void __launch_bounds__(kThreads) mlp_loss_grad_kernel(const uint16_t *w, const uint16_t *x,
-                                                                  const uint8_t *label, const uint32_t *order,
-                                                                  uint32_t n, float *grad, float *loss)
+// Accumulators of a gradient tile added to the global gradient G (row stride
+// ldg), two neighbouring values at a time where G allows.
+__device__ __forceinline__ void flush_grad(float *G, int ldg, int m0, int n0, const float c[4], bool pairs)
+{
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+    float *r0 = G + (m0 + g) * ldg + n0 + 2 * t, *r1 = r0 + 8 * ldg;
+    if (pairs) {
+        atomicAdd(reinterpret_cast<float2 *>(r0), make_float2(c[0], c[1]));
+        atomicAdd(reinterpret_cast<float2 *>(r1), make_float2(c[2], c[3]));
+    } else {
+        atomicAdd(r0, c[0]);
+        atomicAdd(r0 + 1, c[1]);
+        atomicAdd(r1, c[2]);
+        atomicAdd(r1 + 1, c[3]);
+    }
+}
+
+// Rows of `n8` 8-element pieces into padded shared rows: cp.async where the
+// source is 16-byte aligned, else element by element.
+__device__ __forceinline__ void stage_rows(uint16_t *dst, int ld, const uint16_t *src, int rows, int n8, bool vec)
+{
+    for (int i = threadIdx.x; i < rows * n8; i += kTrainThreads) {
+        const int r = i / n8, k = 8 * (i - r * n8);
+        uint16_t *d = dst + r * ld + k;
+        const uint16_t *s = src + (size_t)r * 8 * n8 + k;
+        if (vec)
+            __pipeline_memcpy_async(d, s, 16);
+        else
+            for (int e = 0; e < 8; e++)
+                d[e] = s[e];
+    }
+}
+
+struct TrainSmem {
+    uint16_t w1[NH * LW1], w2[NH * LW2], w3[NO * LW3];
+    uint16_t x[kTile * BX], h1h[kTile * BH], h1l[kTile * BH], h2h[kTile * BH], h2l[kTile * BH];
+    uint16_t zh[kTile * BZ], zl[kTile * BZ], d2h[kTile * BH], d2l[kTile * BH], d1h[kTile * BH], d1l[kTile * BH];
+    float z[kTile * LZ];
+    float b1[NH], b2[NH], b3[NO];
+    float gb1[NH], gb2[NH], gb3[NO];
+    float loss;
+    int cls[kTile];
+};
+static_assert(offsetof(TrainSmem, w2) % 16 == 0 && offsetof(TrainSmem, w3) % 16 == 0 && offsetof(TrainSmem, x) % 16 == 0 &&
+                  offsetof(TrainSmem, h1h) % 16 == 0 && offsetof(TrainSmem, zh) % 16 == 0 && offsetof(TrainSmem, d2h) % 16 == 0,
+              "ldmatrix rows are 16-byte aligned");
+static_assert(kTrainThreads == 512 && kTile == 32 && NH == 64, "sixteen warps, one 16 x 8 tile of a hidden layer each");
+
+__global__ void __launch_bounds__(kTrainThreads, 1) mlp_loss_grad_kernel(const uint16_t *w, const uint16_t *x, const uint8_t *label,
+                                                                     const uint32_t *order, uint32_t n, float *grad, float *loss,
+                                                                     uint32_t vec_w, uint32_t vec_x, uint32_t pairs)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_cls[kTile];
-    __shared__ float s_loss;
-    const NetW m = carve_w(smem, true);
-    float *X = reinterpret_cast<float *>(smem + kWBytes);
-    float *H1 = X + kTile * LX, *H2 = H1 + kTile * LH, *Z = H2 + kTile * LH, *D2 = Z + kTile * LZ, *D1 = D2 + kTile * LH;
-    float *g = D1 + kTile * LH;   // [kP] gradient accumulators, flat parameter order
-    load_weights(w, m, true);
-    for (int i = threadIdx.x; i < kP; i += blockDim.x)
-        g[i] = 0.0f;
-    if (threadIdx.x == 0)
-        s_loss = 0.0f;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kWarps = kThreads / 32, kM = kTile / 16;
+    TrainSmem &m = *reinterpret_cast<TrainSmem *>(smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kTrainThreads / 32;
+    const int m0 = 16 * (warp >> 3), n0 = 8 * (warp & 7);   // this warp's tile of a hidden layer
+    // gradient tiles of this warp: columns n0, every second 16 rows (layers 3
+    // and 2); tiles warp and warp + 16 of 24 (layer 1)
+    float g3[4][4] = {}, g2[2][4] = {}, g1[2][4] = {};
+    // inputs (BF16) and classes (-1 for missing or invalid samples) of a tile
+    const auto load_tile = [&](uint32_t t0) {
+        for (int i = tid; i < kTile * (NI / 8); i += kTrainThreads) {
+            const uint32_t s = i / (NI / 8), k = 8 * (i - s * (NI / 8)), gs = t0 + s;
+            uint16_t *d = m.x + s * BX + k;
+            if (gs >= n) {
+                *reinterpret_cast<uint4 *>(d) = make_uint4(0u, 0u, 0u, 0u);
+            } else {
+                const uint16_t *src = x + (size_t)(order ? order[gs] : gs) * NI + k;
+                if (vec_x)
+                    __pipeline_memcpy_async(d, src, 16);
+                else
+                    for (int e = 0; e < 8; e++)
+                        d[e] = src[e];
+            }
+        }
+        if (tid < kTile) {
+            const uint32_t gs = t0 + tid;
+            int c = -1;
+            if (gs < n) {
+                const uint32_t lab = label[order ? order[gs] : gs];
+                if ((lab & 31u) < (uint32_t)kNumModes)
+                    c = (int)((lab >> 5) * kNumModes + (lab & 31u));
+            }
+            m.cls[tid] = c;
+        }
+    };
     const uint32_t ntiles = (n + kTile - 1) / kTile;
+    load_tile(blockIdx.x * kTile);
+    stage_rows(m.w1, LW1, w + oW1, NH, NI / 8, vec_w);
+    __pipeline_commit();
+    stage_rows(m.w2, LW2, w + oW2, NH, NH / 8, vec_w);
+    __pipeline_commit();
+    stage_rows(m.w3, LW3, w + oW3, NO, NH / 8, vec_w);
+    __pipeline_commit();
+    if (tid < NH) {
+        m.b1[tid] = bf(w[oB1 + tid]);
+        m.b2[tid] = bf(w[oB2 + tid]);
+        m.gb1[tid] = m.gb2[tid] = 0.0f;
+    }
+    if (tid < NO) {
+        m.b3[tid] = bf(w[oB3 + tid]);
+        m.gb3[tid] = 0.0f;
+    }
+    if (tid == 0)
+        m.loss = 0.0f;
+    __pipeline_wait_prior(2);
+    __syncthreads();
     for (uint32_t tt = blockIdx.x; tt < ntiles; tt += gridDim.x) {
-        load_tile(x, label, order, n, tt * kTile, X, s_cls);
+        // forward
+        hidden_tile<NI, true>(m.x, nullptr, BX, m.w1, LW1, m.b1, m.h1h, m.h1l, m0, n0);
+        __pipeline_wait_prior(1);
         __syncthreads();
-        // forward: 16 x 8 output tiles spread over the warps
-        for (int q = warp; q < kM * (NH / 8); q += kWarps)
-            dense_tile<NI, true, true>(X, LX, m.w1, LW1, m.b1, H1, LH, 16 * (q % kM), 8 * (q / kM));
+        hidden_tile<NH, false>(m.h1h, m.h1l, BH, m.w2, LW2, m.b2, m.h2h, m.h2l, m0, n0);
+        __pipeline_wait_prior(0);
         __syncthreads();
-        for (int q = warp; q < kM * (NH / 8); q += kWarps)
-            dense_tile<NH, false, true>(H1, LH, m.w2, LW2, m.b2, H2, LH, 16 * (q % kM), 8 * (q / kM));
+        for (int q = warp; q < 2 * (NO / 8); q += kWarps) {
+            float c[4];
+            const int mt = 16 * (q & 1), nt = 8 * (q >> 1);
+            dense_mma<NH, false>(c, m.h2h, m.h2l, BH, m.w3, LW3, mt, nt);
+            const int g = lane >> 2, nn = nt + 2 * (lane & 3);
+            const float b0 = m.b3[nn], b1 = m.b3[nn + 1];
+            *reinterpret_cast<float2 *>(m.z + (mt + g) * LZ + nn) = make_float2(c[0] + b0, c[1] + b1);
+            *reinterpret_cast<float2 *>(m.z + (mt + g + 8) * LZ + nn) = make_float2(c[2] + b0, c[3] + b1);
+        }
         __syncthreads();
-        for (int q = warp; q < kM * (NO / 8); q += kWarps)
-            dense_tile<NH, false, false>(H2, LH, m.w3, LW3, m.b3, Z, LZ, 16 * (q % kM), 8 * (q / kM));
-        __syncthreads();
-        // softmax cross-entropy; Z becomes d loss / d z
+        // softmax cross-entropy; z becomes d loss / d z, also as BF16 terms
         for (int s = warp; s < kTile; s += kWarps) {
-            float *z = Z + s * LZ;
-            const int y = s_cls[s];
+            float *z = m.z + s * LZ;
+            const int y = m.cls[s];
             float zmax = -INFINITY;
             for (int j = lane; j < NO; j += 32)
                 zmax = fmaxf(zmax, z[j]);
@@ -488,51 +631,93 @@ __global__ void __launch_bounds__(kThreads) mlp_loss_grad_kernel(const uint16_t 
             for (int d = 16; d > 0; d >>= 1)
                 den += __shfl_xor_sync(kFull, den, d);
             if (lane == 0 && y >= 0)
-                atomicAdd(&s_loss, logf(den) + zmax - z[y]);
+                atomicAdd(&m.loss, logf(den) + zmax - z[y]);
             __syncwarp();
-            for (int j = lane; j < NO; j += 32)
-                z[j] = y >= 0 ? expf(z[j] - zmax) / den - (j == y ? 1.0f : 0.0f) : 0.0f;
+            for (int j = lane; j < NO; j += 32) {
+                const float d = y >= 0 ? expf(z[j] - zmax) / den - (j == y ? 1.0f : 0.0f) : 0.0f;
+                z[j] = d;
+                const uint16_t h = to_bf(d);
+                m.zh[s * BZ + j] = h;
+                m.zl[s * BZ + j] = to_bf(d - bf(h));
+            }
         }
         __syncthreads();
-        // layer 3: gW3 += dz^T h2 (112 x 64), gb3; d2 = (dz W3) relu'(h2)
-        for (int q = warp; q < (NO / 16) * (NH / 8); q += kWarps)
-            grad_tile<false>(Z, LZ, H2, LH, g + oW3, NH, 16 * (q % (NO / 16)), 8 * (q / (NO / 16)));
-        for (int q = warp; q < kM * (NH / 8); q += kWarps)
-            delta_tile<NO>(Z, LZ, m.w3t, LW3T, H2, LH, D2, LH, 16 * (q % kM), 8 * (q / kM));
-        for (int j = threadIdx.x; j < NO; j += kThreads) {
+        // layer 3: gW3 += dz^T h2, gb3; d2 = (dz W3) relu'(h2)
+        {
+            uint32_t bh[2][2], bl[2][2];
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                load_bt(bh[k], m.h2h, BH, n0, 16 * k);
+                load_bt(bl[k], m.h2l, BH, n0, 16 * k);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (m0 + 32 * i < NO)
+                    grad_acc<false>(g3[i], m.zh, m.zl, BZ, bh, bl, m0 + 32 * i);
+        }
+        delta_tile<NO>(m.zh, m.zl, BZ, m.w3, LW3, m.h2h, m.d2h, m.d2l, m.gb2, m0, n0);
+        if (tid < NO) {
             float a = 0.0f;
             for (int s = 0; s < kTile; s++)
-                a += Z[s * LZ + j];
-            g[oB3 + j] += a;
+                a += m.z[s * LZ + tid];
+            m.gb3[tid] += a;
         }
         __syncthreads();
-        // layer 2: gW2 += d2^T h1 (64 x 64), gb2; d1 = (d2 W2) relu'(h1)
-        for (int q = warp; q < (NH / 16) * (NH / 8); q += kWarps)
-            grad_tile<false>(D2, LH, H1, LH, g + oW2, NH, 16 * (q % (NH / 16)), 8 * (q / (NH / 16)));
-        for (int q = warp; q < kM * (NH / 8); q += kWarps)
-            delta_tile<NH>(D2, LH, m.w2t, LW2T, H1, LH, D1, LH, 16 * (q % kM), 8 * (q / kM));
-        for (int j = threadIdx.x; j < NH; j += kThreads) {
-            float a = 0.0f;
-            for (int s = 0; s < kTile; s++)
-                a += D2[s * LH + j];
-            g[oB2 + j] += a;
+        // layer 2: gW2 += d2^T h1; d1 = (d2 W2) relu'(h1)
+        {
+            uint32_t bh[2][2], bl[2][2];
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                load_bt(bh[k], m.h1h, BH, n0, 16 * k);
+                load_bt(bl[k], m.h1l, BH, n0, 16 * k);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+                grad_acc<false>(g2[i], m.d2h, m.d2l, BH, bh, bl, m0 + 32 * i);
+        }
+        delta_tile<NH>(m.d2h, m.d2l, BH, m.w2, LW2, m.h1h, m.d1h, m.d1l, m.gb1, m0, n0);
+        __syncthreads();
+        // layer 1: gW1 += d1^T x
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            const int q = warp + 16 * i, mt = q / (NI / 8), nt = q - mt * (NI / 8);
+            if (q < (NH / 16) * (NI / 8)) {
+                uint32_t bx[2][2];
+#pragma unroll
+                for (int k = 0; k < 2; k++)
+                    load_bt(bx[k], m.x, BX, 8 * nt, 16 * k);
+                grad_acc<true>(g1[i], m.d1h, m.d1l, BH, bx, bx, 16 * mt);
+            }
         }
         __syncthreads();
-        // layer 1: gW1 += d1^T x (64 x 48), gb1
-        for (int q = warp; q < (NH / 16) * (NI / 8); q += kWarps)
-            grad_tile<true>(D1, LH, X, LX, g + oW1, NI, 16 * (q % (NH / 16)), 8 * (q / (NH / 16)));
-        for (int j = threadIdx.x; j < NH; j += kThreads) {
-            float a = 0.0f;
-            for (int s = 0; s < kTile; s++)
-                a += D1[s * LH + j];
-            g[oB1 + j] += a;
+        if (tt + gridDim.x < ntiles) {
+            load_tile((tt + gridDim.x) * kTile);
+            __pipeline_commit();
+            __pipeline_wait_prior(0);
+            __syncthreads();
         }
-        __syncthreads();
     }
-    for (int i = threadIdx.x; i < kP; i += blockDim.x)
-        atomicAdd(&grad[i], g[i]);
-    if (threadIdx.x == 0)
-        atomicAdd(loss, s_loss);
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+        if (m0 + 32 * i < NO)
+            flush_grad(grad + oW3, NH, m0 + 32 * i, n0, g3[i], pairs);
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+        flush_grad(grad + oW2, NH, m0 + 32 * i, n0, g2[i], pairs);
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        const int q = warp + 16 * i, mt = q / (NI / 8), nt = q - mt * (NI / 8);
+        if (q < (NH / 16) * (NI / 8))
+            flush_grad(grad + oW1, NI, 16 * mt, 8 * nt, g1[i], pairs);
+    }
+    if (tid < NH) {
+        atomicAdd(&grad[oB1 + tid], m.gb1[tid]);
+        atomicAdd(&grad[oB2 + tid], m.gb2[tid]);
+    }
+    if (tid < NO)
+        atomicAdd(&grad[oB3 + tid], m.gb3[tid]);
+    if (tid == 0)
+        atomicAdd(loss, m.loss);
 }
 
 // Inference: each warp takes 16 samples at a time through the three layers
@@ -544,8 +729,8 @@ __global__ void __launch_bounds__(kThreads) mlp_predict_kernel(const uint16_t *w
                                                                 const uint32_t *index, uint8_t *label)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const NetW m = carve_w(smem, false);
-    load_weights(w, m, false);
+    const NetW m = carve_w(smem);
+    load_weights(w, m);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *X = reinterpret_cast<float *>(smem + kWBytes) + warp * kPredWarpFloats;
@@ -716,11 +901,12 @@ RLFC_API int rlfc_mlp_loss_grad(const uint16_t *d_w, const uint16_t *d_x, const 
         return RLFC_E_RANGE;
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const size_t smem = kWBytes + sizeof(float) * (kTileFloats + kP);
+    const size_t smem = sizeof(TrainSmem);
+    const uint32_t vec_w = ((uintptr_t)d_w & 15u) == 0, vec_x = ((uintptr_t)d_x & 15u) == 0, pairs = ((uintptr_t)d_grad & 7u) == 0;
     cudaError_t e = cudaFuncSetAttribute(mlp_loss_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return cuda_fail(e, "rlfc_mlp_loss_grad");
-    { TraceScope trace_("mlp_loss_grad_kernel", st); mlp_loss_grad_kernel<<<net_grid((uint32_t)n, sm_count()), kThreads, smem, st>>>(d_w, d_x, d_label, d_order, (uint32_t)n, d_grad, d_loss); }
+    { TraceScope trace_("mlp_loss_grad_kernel", st); mlp_loss_grad_kernel<<<net_grid((uint32_t)n, sm_count()), kTrainThreads, smem, st>>>(d_w, d_x, d_label, d_order, (uint32_t)n, d_grad, d_loss, vec_w, vec_x, pairs); }
     e = cudaGetLastError();
     return e == cudaSuccess ? RLFC_OK : cuda_fail(e, "rlfc_mlp_loss_grad");
 }
