@@ -108,6 +108,31 @@ __device__ __forceinline__ void decode_block_pairs(const uint32_t *rec, uint32_t
     }
 }
 
+// Reads the 18-bit headers of a record one after the other through a 64-bit
+// window, a word at a time.
+struct HeaderReader {
+    const uint32_t *next;
+    uint64_t win;
+    uint32_t have;
+    __device__ __forceinline__ HeaderReader(const uint32_t *rec, uint32_t MW)
+    {
+        next = rec + MW;
+        win = *next++;
+        have = 32;
+    }
+    __device__ __forceinline__ uint32_t take()
+    {
+        if (have < (uint32_t)kHdrBits) {
+            win |= (uint64_t)*next++ << have;
+            have += 32;
+        }
+        const uint32_t h = (uint32_t)win & 0x3FFFFu;
+        win >>= kHdrBits;
+        have -= kHdrBits;
+        return h;
+    }
+};
+
 __device__ __forceinline__ uint32_t clamp_biased_u8(uint32_t x)
 {
     // each biased half into [2^14, 2^14 + 255]: its low byte is then the value

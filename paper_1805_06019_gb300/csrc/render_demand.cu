@@ -57,31 +57,6 @@ struct Rect {
 
 extern __shared__ __align__(16) uint32_t g_smem[];
 
-// Reads the 18-bit headers of a record one after the other through a 64-bit
-// window, a word at a time.
-struct HeaderReader {
-    const uint32_t *next;
-    uint64_t win;
-    uint32_t have;
-    __device__ __forceinline__ HeaderReader(const uint32_t *rec, uint32_t MW)
-    {
-        next = rec + MW;
-        win = *next++;
-        have = 32;
-    }
-    __device__ __forceinline__ uint32_t take()
-    {
-        if (have < (uint32_t)kHdrBits) {
-            win |= (uint64_t)*next++ << have;
-            have += 32;
-        }
-        const uint32_t h = (uint32_t)win & 0x3FFFFu;
-        win >>= kHdrBits;
-        have -= kHdrBits;
-        return h;
-    }
-};
-
 template <bool kNative>
 __global__ void __launch_bounds__(kThreads, 4) render_demand_kernel(const Args a)
 {
