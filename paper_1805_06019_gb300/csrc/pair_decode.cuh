@@ -181,15 +181,15 @@ __device__ __forceinline__ void row_to_rgb(const uint2 y, const uint2 co, const 
 
 // Bytes [0, len) of a strip row (`src`, word-aligned shared memory with a
 // chunk of readable padding on each side) to `row`, whatever its alignment:
-// lane `ch` of eight takes the 16-byte aligned chunk ch of the destination,
+// the caller's lanes take its 16-byte aligned chunks ch = 0, 1, ... (len + 30) / 16 - 1,
 // which begins at source byte 16 ch - (row & 15); five words funnel-shifted to
 // four make it, and only the first and last chunk of the row, shared with the
-// neighbouring strips, go out as words and bytes.  len <= 112.
+// neighbouring strips, go out in smaller pieces.
 //
 // What bounds it: instruction issue (about 25 instructions for up to 512
-// bytes; the edges another 40).  The 15 x 15 x 625 x 434 decode takes 0.250 ms
+// bytes; the edges another 30).  The 15 x 15 x 625 x 434 decode takes 0.249 ms
 // with it; with single bytes or 4-byte words, each placed by divisions by the
-// row length, it took 0.695 ms.
+// row length, it took 0.695 ms; with the edges as single bytes, 0.255.
 __device__ __forceinline__ void store_row_unaligned(uint8_t *row, const uint32_t *src, uint32_t len, uint32_t ch)
 {
     const int b0 = (int)(16u * ch) - (int)((uintptr_t)row & 15u);
@@ -215,12 +215,30 @@ __device__ __forceinline__ void store_row_unaligned(uint8_t *row, const uint32_t
         p4[2] = y2;
     if (lo <= 12 && hi >= 16)
         p4[3] = y3;
-    const uint8_t *sb = reinterpret_cast<const uint8_t *>(src) + b0;
-    const int up = (lo + 3) & ~3;
-    for (int j = lo; j < min(hi, up); j++)
-        p[j] = sb[j];
-    for (int j = max(hi & ~3, up); j < hi; j++)
-        p[j] = sb[j];
+    // the boundary words: up to 3 bytes in front of a word boundary, up to 3
+    // behind one, in pieces of their own alignment; bytes [lo, hi) of one word
+    // where the row is that short
+    if ((lo >> 2) == (hi >> 2)) {
+        const uint8_t *sb = reinterpret_cast<const uint8_t *>(src) + b0;
+        for (int j = lo; j < hi; j++)
+            p[j] = sb[j];
+        return;
+    }
+    if (lo & 3) {
+        const uint32_t a = lo < 8 ? (lo < 4 ? y0 : y1) : (lo < 12 ? y2 : y3);
+        if (lo & 1)
+            p[lo] = (uint8_t)(a >> (8 * (lo & 3)));
+        if ((lo & 3) != 3)
+            *reinterpret_cast<uint16_t *>(p + (lo & ~3) + 2) = (uint16_t)(a >> 16);
+    }
+    if (hi & 3) {
+        const uint32_t a = hi < 8 ? (hi < 4 ? y0 : y1) : (hi < 12 ? y2 : y3);
+        const int w = hi & ~3;
+        if (hi & 2)
+            *reinterpret_cast<uint16_t *>(p + w) = (uint16_t)a;
+        if (hi & 1)
+            p[hi - 1] = (uint8_t)(a >> (8 * ((hi - 1) & 3)));
+    }
 }
 
 }  // namespace rlfc
