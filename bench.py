@@ -44,22 +44,22 @@ UNIT = "Mpix/s"
 # capture of the same kernel build on this workload (config, tau, views,
 # kernel); a kernel missing here reports null
 TRAFFIC_PER_LAUNCH = {
-    # render_native_kernel, first timed step of `bench.py --steps 2 --warmup 1` (ncu one-pass
-    # dram__bytes_read.sum 86.56 MB + dram__bytes_write.sum 3.09 GB)
-    ("plain", 4, 1000, "render_native_kernel"): 86_560_000 + 3_090_000_000,
+    # render_native_kernel, first timed step of `bench.py --steps 2 --warmup 3` (ncu one-pass
+    # dram__bytes_read.sum 127.74 MB + dram__bytes_write.sum 3.08 GB)
+    ("plain", 4, 1000, "render_native_kernel"): 127_742_720 + 3_083_778_560,
     # decode_all_kernel on the 17x17x1024^2 light field at tau 4 (ncu one-pass, third launch:
-    # dram__bytes_read.sum 100.21 MB + dram__bytes_write.sum 853.10 MB; the rest of the
+    # dram__bytes_read.sum 100.72 MB + dram__bytes_write.sum 853.53 MB; the rest of the
     # 909 MB of output is still in L2 when the kernel ends)
-    ("batching", 4, 0, "decode_all_kernel"): 100_210_000 + 853_100_000,
+    ("batching", 4, 0, "decode_all_kernel"): 100_717_824 + 853_529_088,
 }
 
 # smsp__inst_executed.sum of one launch (warp instructions), from the same kind
-# of one-pass ncu capture (`--metrics smsp__inst_executed.sum ... -s 3 -c 3`
-# on `bench.py --steps 2 --warmup 1`); the kernels are integer and
+# of one-pass ncu capture (`--metrics smsp__inst_executed.sum ... -s 3 -c 1`
+# on `bench.py --steps 2 --warmup 3`); the kernels are integer and
 # conversion work bound by instruction issue more than by DRAM
 INSTR_PER_LAUNCH = {
-    ("plain", 4, 1000, "render_native_kernel"): 1_072_146_688,
-    ("batching", 4, 0, "decode_all_kernel"): 458_440_390,
+    ("plain", 4, 1000, "render_native_kernel"): 724_261_584,
+    ("batching", 4, 0, "decode_all_kernel"): 430_273_741,
 }
 # issue peak: 152 SMs x 4 schedulers x one warp instruction per cycle at the
 # 2070 MHz maximum SM clock
@@ -354,7 +354,7 @@ def _extra_parts(rlfc, torch, args, p, tau, st, out_lf, flush, peak, world):
             "config": chosen, "identical_to_per_request": same,
             "note": "persistent binned kernel, autotuned, replayed as a CUDA graph"}
         out["per_request_1e6"] = {"ms": per_req, "requests_per_s": n / (per_req * 1e-3),
-                                  "mpix_s": 16 * n / (per_req * 1e-3) / 1e6, "note": "one warp per request"}
+                                  "mpix_s": 16 * n / (per_req * 1e-3) / 1e6, "note": "one rlfc_decode_blocks call (a thread per request and channel)"}
         out["batched_speedup_vs_per_request"] = per_req / g_ms
         bt.close()
         s_b.close()
@@ -679,7 +679,7 @@ def _stream_location_words(data: bytes):
 def run_batching(args):
     """10^6 uniform random (view, location) block requests per launch on the
     17 x 17 x 1024^2 light field: the persistent binned kernel (autotuned,
-    eager and replayed as a CUDA graph) against one warp per request, plus a
+    eager and replayed as a CUDA graph) against one rlfc_decode_blocks call, plus a
     full decode of the same light field."""
     import torch
     from paper_1805_06019_gb300 import rlfc

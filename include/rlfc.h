@@ -160,7 +160,8 @@ RLFC_API int rlfc_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, co
  * view (i, j) it samples (s + d (i - u), t + d (j - v)) bilinearly with
  * clamp-to-edge, and the four views are blended bilinearly in (u, v).
  * d_out receives n * out_h * out_w * 3 floats (RGB in [0, 1]), view-major.
- * At native size a call of four or more cameras first decodes the neighbour
+ * A call of three or more cameras (and of 400 000 or more pixels of the
+ * views' own size in all) first decodes the neighbour
  * views they need into a transient device buffer (stream-ordered
  * allocation on cuda_stream, released before the call's work completes:
  * 4 * H * (W rounded up to 32) bytes per needed view, at most min(views, 4n)
