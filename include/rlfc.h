@@ -167,8 +167,8 @@ RLFC_API int rlfc_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, co
  * 4 * H * (W rounded up to 32) bytes per needed view, at most min(views, 4n)
  * of them, and about 200 bytes per camera); if that allocation fails the
  * call decodes on demand instead.  The loaded stream's own memory pool keeps
- * what its calls used for the next ones, up to the packed size of all its
- * views and at most 512 MiB, until rlfc_free_stream.  Results do not depend
+ * what its calls used for the next ones, up to four times the packed size of
+ * all its views (64 MiB at least, 4 GiB at most), until rlfc_free_stream.  Results do not depend
  * on the path or on the other views of the call.
  * Errors: RLFC_E_INVALID_ARG, RLFC_E_RANGE, RLFC_E_UNSUPPORTED, RLFC_E_CUDA.
  */

@@ -302,11 +302,14 @@ void free_device(rlfc_stream *s)
     s->d_view_anc = nullptr;
 }
 
-// The pool keeps what a render call used for the next one, up to the packed
-// views of the whole light field and at most this much.  (The device's
-// default pool gives everything back at each synchronisation: a call after
-// one then maps its memory anew, 180 us for one view and 400 us for 85 MB.)
-constexpr uint64_t kScratchKeep = 512ull << 20;
+// The pool keeps what render calls used for the next ones: up to four calls'
+// largest scratch (the packed views of the whole light field each), within
+// these bounds.  (The device's default pool gives everything back at each
+// synchronisation: a call after one then maps its memory anew, 180 us for one
+// view and 400 us for 85 MB.  A bound below what the calls in flight on a
+// server's four streams hold does the same to them: at 80 000 small views per
+// second 0.8 ms of latency instead of 0.1.)
+constexpr uint64_t kScratchKeepLeast = 64ull << 20, kScratchKeepMost = 4ull << 30;
 
 void make_pool(rlfc_stream *s)
 {
@@ -315,7 +318,8 @@ void make_pool(rlfc_stream *s)
     props.handleTypes = cudaMemHandleTypeNone;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = s->device;
-    uint64_t keep = std::min<uint64_t>(kScratchKeep, 4ull * packed_pitch(s->info.W) * s->info.H * s->tab.n_views + (1u << 20));
+    const uint64_t call = 4ull * packed_pitch(s->info.W) * s->info.H * s->tab.n_views + (1u << 20);
+    uint64_t keep = std::clamp<uint64_t>(4 * call, kScratchKeepLeast, kScratchKeepMost);
     if (cudaMemPoolCreate(&s->pool, &props) != cudaSuccess ||
         cudaMemPoolSetAttribute(s->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
         if (s->pool)
