@@ -466,6 +466,12 @@ struct DevBuf {
             arena_used = at + bytes;
             return cudaSuccess;
         }
+        return alloc_own(p, count);
+    }
+    // a buffer of its own
+    template <typename T>
+    cudaError_t alloc_own(T **p, size_t count)
+    {
         cudaError_t e = cudaMalloc((void **)p, count * sizeof(T) + 16);
         if (e == cudaSuccess)
             ptrs.push_back((void *)*p);
@@ -485,21 +491,24 @@ size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 }  // namespace
 
-// Upper bound of the device scratch encode_gpu carves for these parameters
-// (every buffer rounded up to 256 bytes, records at their largest possible
-// size); 0 when the parameters are invalid.
-size_t encode_scratch_bound(const rlfc_enc_params *p)
+namespace {
+
+// Upper bounds of the device scratch that encode_gpu carves for these
+// parameters (every buffer rounded up to 256 bytes): everything but the
+// records, and the records at their largest possible size; false when the
+// parameters are invalid.
+bool scratch_bounds(const rlfc_enc_params *p, uint64_t &fixed, uint64_t &records)
 {
     if (!p || p->B != 4 || p->U < 1 || p->V < 1 || (uint64_t)p->U * p->V > 16383 || p->W < 1 || p->H < 1 ||
         p->W > 65536 || p->H > 65536 || p->L < 2 || p->L > (uint32_t)kMaxLevels)
-        return 0;
+        return false;
     const uint32_t L = p->L;
     std::vector<uint64_t> cnt(L);
     uint64_t Gu = p->U, Gv = p->V;
     cnt[0] = Gu * Gv;
     for (uint32_t l = 1; l < L; l++) {
         if (p->c[l] < 1)
-            return 0;
+            return false;
         Gu = (Gu + p->c[l] - 1) / p->c[l];
         Gv = (Gv + p->c[l] - 1) / p->c[l];
         cnt[l] = Gu * Gv;
@@ -537,8 +546,19 @@ size_t encode_scratch_bound(const rlfc_enc_params *p)
     add(sizeof(void *) * L);
     add(sizeof(void *) * L);
     const uint64_t MW = (S + 31) / 32;
+    fixed = total;
+    total = 0;
     add(4 * (3 * nloc * (MW + (S * (kHdrBits + 160) + 31) / 32) + 1));
-    return (size_t)total;
+    records = total;
+    return true;
+}
+
+}  // namespace
+
+size_t encode_scratch_bound(const rlfc_enc_params *p)
+{
+    uint64_t fixed = 0, records = 0;
+    return scratch_bounds(p, fixed, records) ? (size_t)(fixed + records) : 0;
 }
 
 int encode_gpu(const rlfc_enc_params *p, const uint8_t *d_rgb, cudaStream_t st, std::vector<uint8_t> &out,
@@ -598,6 +618,15 @@ int encode_gpu(const rlfc_enc_params *p, const uint8_t *d_rgb, cudaStream_t st, 
     buf.arena = arena;
     buf.arena_size = arena_size;
     cudaError_t e;
+    if (!arena) {
+        // one allocation for everything but the records (a dozen of them, and
+        // as many frees, took 0.25 ms)
+        uint64_t fixed = 0, records = 0;
+        scratch_bounds(p, fixed, records);
+        if ((e = buf.alloc_own(&buf.arena, fixed)) != cudaSuccess)
+            return cuda_fail(e, "encoder allocation");
+        buf.arena_size = fixed;
+    }
     std::vector<int16_t *> img(L, nullptr), rec(L, nullptr);
     std::vector<uint8_t *> kmode(L, nullptr);
     for (uint32_t l = 0; l < L; l++) {
@@ -761,7 +790,7 @@ int encode_gpu(const rlfc_enc_params *p, const uint8_t *d_rgb, cudaStream_t st, 
         set_error("stream larger than 16 GiB");
         return RLFC_E_RANGE;
     }
-    if ((e = buf.alloc(&d_rec, total + 1)) != cudaSuccess)
+    if ((e = arena ? buf.alloc(&d_rec, total + 1) : buf.alloc_own(&d_rec, total + 1)) != cudaSuccess)
         return cuda_fail(e, "encoder allocation");
     cudaMemcpyAsync(d_off, offsets.data(), 4ull * offsets.size(), cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(d_rec, 0, 4ull * total, st);   // shared words are ORed
