@@ -77,7 +77,7 @@ __host__ __device__ __forceinline__ int window_rows(int oymin, int oymax) { retu
 
 // One CTA.  What bounds it: its own latency (a few passes over the cameras and
 // the grid); it replaces four small launches and the camera scan that every
-// tile's CTA did, and takes 6 us for 1000 cameras on a 9 x 9 grid.
+// tile's CTA did, and takes 16 us for 1000 cameras on a 9 x 9 grid, 9 for 24.
 __global__ void __launch_bounds__(kPlanThreads) render_plan_kernel(const Plan a)
 {
     extern __shared__ uint32_t sm[];
@@ -528,8 +528,9 @@ __global__ void __launch_bounds__(kThreads, 3) render_native_kernel(const Args a
 }
 
 // Any output size: a thread per output pixel samples the decoded views through
-// the caches.  What bounds it: instruction issue (about 350 instructions per
-// pixel for 16 samples, their weights and coordinates).
+// the caches.  What bounds it: instruction issue (16 samples, their weights and
+// coordinates per pixel); eight 800 x 600 views take 79 us, and with the
+// decode of their neighbours 0.14 ms (1.0 with a warp per block of every tile).
 constexpr int kSX = 32, kSY = 8;
 
 __global__ void __launch_bounds__(kSX * kSY) render_sampled_kernel(const Args a, const float *uv, const float *disp, uint32_t out_w,
