@@ -48,10 +48,12 @@ static __device__ const DecodeTables g_tables = make_tables();
 //
 // The 16 values come out dequantised and biased, two to a word (value 2j in
 // the low half of out[j], 2j + 1 in the high half), and are built two at a
-// time: every term of (digit << b | low part) << shift + (min << shift) +
-// 2^14 is non-negative and the sum of each half stays below 2^15 (the
-// loader's range check), so the pair needs one 32-bit multiply-add per term
-// and no carry crosses the halves.
+// time: a pair stands for low half + 2^16 * high half modulo 2^32, and every
+// term of (digit << b | low part) << shift + (min << shift) + 2^14 enters it
+// as first + 2^16 * second, the possibly negative min included.  The terms of
+// a half may leave its 16 bits (a minimum far below the values that the block
+// holds); their sums do not (the loader bounds the values), so the result is
+// exact, with one 32-bit multiply-add per term.
 // Digits (trit and quint blocks) come first in the payload: the groups are
 // split by the base-3 / base-5 tables (digit v at bits 3v of a 64-bit word).
 // The low parts of block row rr (values 4rr .. 4rr + 3, 4b <= 40 bits) sit
@@ -64,7 +66,7 @@ __device__ __forceinline__ void decode_block_pairs(const uint32_t *rec, uint32_t
     const uint32_t scale = 1u << (q + ((hdr >> 5) & 3u));
     const int32_t mn = ((int32_t)(hdr << 14)) >> 21;   // header bits 7..17, sign-extended
     const uint32_t base = (uint32_t)mn * scale + 0x4000u;
-    const uint32_t base2 = base | (base << 16);
+    const uint32_t base2 = base + (base << 16);
     const uint32_t m2 = ((1u << b) - 1u) * 0x10001u;   // the low-part mask in both halves
     const uint32_t sb = scale << b;
     uint64_t dw = 0;   // digit v at bits 3v
