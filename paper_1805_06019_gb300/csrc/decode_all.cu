@@ -676,7 +676,9 @@ int launch_decode(const rlfc_stream *s, uint8_t *d_out, const uint8_t *needed, c
         return RLFC_E_UNSUPPORTED;
     }
     auto kern = off16 ? decode_all_kernel<kPacked, uint16_t> : decode_all_kernel<kPacked, uint32_t>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the same limit for every call: the attribute belongs to the kernel, and
+    // a smaller one set for another thread's light field would refuse this launch)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
     if (e != cudaSuccess)
         return cuda_fail(e, "decode_all: shared memory attribute");
     dim3 grid((a.nlx + kNL - 1) / kNL, s->info.nloc_y);

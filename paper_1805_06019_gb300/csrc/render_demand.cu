@@ -353,7 +353,9 @@ int launch_render_demand(const rlfc_stream *s, const float *d_uv, const float *d
         return RLFC_E_UNSUPPORTED;
     auto kern = native ? render_demand_kernel<true> : render_demand_kernel<false>;
     cudaError_t e;
-    if (smem > 40u * 1024u && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    // (the same limit for every call: the attribute belongs to the kernel, and
+    // a smaller one set for another thread's light field would refuse this launch)
+    if (smem > 40u * 1024u && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost)) != cudaSuccess)
         return cuda_fail(e, "render_demand: shared memory attribute");
     { TraceScope trace_("render_demand_kernel", st); kern<<<dim3((uint32_t)n_tiles, n), kThreads, smem, st>>>(a); }
     if ((e = cudaGetLastError()) != cudaSuccess)

@@ -35,6 +35,11 @@ constexpr int kPitch = 18;                 // quads of a window row: a compile-t
 // cameras and the staged output rows (fewer bytes for 8-bit output)
 constexpr uint32_t kWinBytes = 46 * 1024, kWinBytesU8 = 64 * 1024;
 constexpr int kPlanThreads = 1024;
+constexpr uint32_t kPlanViews = 32 * kPlanThreads;   // views at most: a mask word per thread
+constexpr uint32_t plan_bytes(uint32_t n_cells, uint32_t n_views) { return 4u * (n_cells + 1 + 2 * ((n_views + 31) / 32)) + 2u * n_cells; }
+// (one limit for every call: the attribute that sets it belongs to the kernel,
+// not to the call; a grid has no more cells than views)
+constexpr uint32_t kPlanSmemMost = plan_bytes(kPlanViews, kPlanViews);
 
 // One camera: the four neighbours' stencil weights (blend weight / 255 times
 // the bilinear weights) and integer shifts.
@@ -581,7 +586,7 @@ int launch_render_decoded(const rlfc_stream *s, const float *d_uv, const float *
     a.n_tiles = a.tiles_x * ((s->info.H + kTH - 1) / kTH);
     const uint32_t stiles_x = (out_w + kSX - 1) / kSX;
     const uint64_t stiles = (uint64_t)stiles_x * ((out_h + kSY - 1) / kSY);
-    if (n_views > 32u * kPlanThreads || (uint64_t)a.n_tiles * n >= (1ull << 32) - (1u << 20) || stiles >= (1ull << 31))
+    if (n_views > kPlanViews || (uint64_t)a.n_tiles * n >= (1ull << 32) - (1u << 20) || stiles >= (1ull << 31))
         return RLFC_E_UNSUPPORTED;
     // one stream-ordered block: the plan, then a slot per needed view (a
     // camera needs at most four views, so min(views, 4n) slots suffice)
@@ -614,12 +619,12 @@ int launch_render_decoded(const rlfc_stream *s, const float *d_uv, const float *
     a.bulk = d_out8 ? ((uintptr_t)d_out8 & 15u) == 0 && s->info.W % 16 == 0 : ((uintptr_t)d_out & 15u) == 0 && s->info.W % 4 == 0;
     const uint32_t win_bytes = p.win_bytes = d_out8 ? kWinBytesU8 : kWinBytes;
     auto kern = d_out8 ? render_native_kernel<true> : render_native_kernel<false>;
-    const uint32_t plan_smem = 4u * (n_cells + 1 + 2 * ((n_views + 31) / 32)) + 2u * n_cells;
+    const uint32_t plan_smem = plan_bytes(n_cells, n_views);
     int sms = 0, per_sm = 0, rc = RLFC_OK;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes)) != cudaSuccess ||
         (plan_smem > 40u * 1024u && (e = cudaFuncSetAttribute(render_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                              (int)plan_smem)) != cudaSuccess) ||
+                                                              (int)kPlanSmemMost)) != cudaSuccess) ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device)) != cudaSuccess ||
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, win_bytes)) != cudaSuccess)
         rc = cuda_fail(e, "render: launch configuration");
