@@ -166,7 +166,9 @@ RLFC_API int rlfc_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, co
  * allocation on cuda_stream, released before the call's work completes:
  * 4 * H * (W rounded up to 32) bytes per needed view, at most min(views, 4n)
  * of them, and about 200 bytes per camera); if that allocation fails the
- * call decodes on demand instead.  The loaded stream's own memory pool keeps
+ * call decodes on demand instead.  Outputs much smaller than the views of a
+ * large light field (thumbnails) decode just the pixels they sample, without
+ * scratch, where that is estimated to be the faster.  The loaded stream's own memory pool keeps
  * what its calls used for the next ones, up to four times the packed size of
  * all its views (64 MiB at least, 4 GiB at most), until rlfc_free_stream.  Results do not depend
  * on the path or on the other views of the call.

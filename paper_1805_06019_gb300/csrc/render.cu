@@ -9,9 +9,8 @@
 // U - 2), i1 = i0 + 1 are blended with weights 1 - fu, fu, and the same in v.
 //
 // This file routes a call to the renderers of render_windows.cu and
-// render_demand.cu, and holds the kernel of last resort (heavy downscaling,
-// whose footprints do not fit shared memory, when there is no scratch to
-// decode into): each thread decodes the pixels it samples one by one.
+// render_demand.cu, and holds the renderer of thumbnails (outputs much smaller
+// than the views): each thread decodes the pixels that it samples, one by one.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -116,17 +115,46 @@ __global__ void __launch_bounds__(256) render_direct_kernel(const Args a)
     store_rgb(a.out, a.out8, ((size_t)n * a.out_h + y) * a.out_w + x, acc[0], acc[1], acc[2]);
 }
 
+// Times of a call at another size than the views' by the three paths, in us,
+// fitted to 500 calls (5 x 5 x 256^2 to 17 x 17 x 2048^2 and 5 x 5 x 4096^2, 1
+// to 1000 cameras, outputs of a half to a 128th of the views' width; median
+// errors 4 % decoded, 16 % direct).  A thumbnail samples a few pixels of many
+// blocks: pixel by pixel it costs its header walks, while the other paths
+// decode every block in view.  Measured, one camera, direct / decoded first:
+// 9 x 9 x 2048^2 at 128 x 128 163 / 485; 17 x 17 x 2048^2 at 64 x 64 274 / 1122;
+// 5 x 5 x 4096^2 at 256 x 256 134 / 1405, at 682 x 682 435 / 751 (on demand);
+// and where it does not pay: 17 x 17 x 1024^2 at 128 x 128 377 / 136 (on
+// demand), 9 x 9 x 512^2 at 32 x 32 170 / 54, 1000 cameras of 9 x 9 x 1024^2 at
+// 32 x 32 3171 / 334.
+struct Estimate {
+    double n, nodes;                   // cameras, tree nodes
+    double src, stream, needed, px;    // megapixels of a view, megabytes of records, megapixels of the needed views and of the output
+    Estimate(const rlfc_stream &s, uint32_t out_w, uint32_t out_h, uint32_t cams)
+        : n(cams), nodes(s.tab.S), src(1e-6 * s.info.W * s.info.H), stream(4e-6 * s.record_words),
+          needed(src * std::min<double>(s.tab.n_views, 4.0 * n)), px(1e-6 * out_w * out_h * n)
+    {
+    }
+    double decoded() const { return 25 + src * (49 + 0.41 * nodes) + 1.35 * stream + 1.13 * needed + 25 * px; }
+    double demand() const { return 20 + n * src * (36 + 0.22 * nodes); }
+    double direct() const { return 90 + nodes * (n < 3 ? 0.7 : 1.5) + px * (700 + 12 * nodes); }
+};
+
 }  // namespace
 
 int launch_render(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t out_w,
                   uint32_t out_h, uint32_t n, float *d_out, cudaStream_t st, uint8_t *d_out8)
 {
     const bool first = n >= kDecodeFirstViews && (uint64_t)n * s->info.W * s->info.H >= kDecodeFirstPixels;
+    const bool native = out_w == s->info.W && out_h == s->info.H;
+    const Estimate cost(*s, out_w, out_h, n);
     for (int turn = 0; turn < 2; turn++) {
         // the other path where the first cannot run: no scratch to decode
         // into, or a tile's footprint too large for shared memory
-        const int rc = (turn == 0) == first ? launch_render_decoded(s, d_uv, d_disp, out_w, out_h, n, d_out, st, d_out8)
-                                            : launch_render_demand(s, d_uv, d_disp, out_w, out_h, n, d_out, st, d_out8);
+        const bool decode = (turn == 0) == first;
+        if (!native && cost.direct() < 0.95 * (decode ? cost.decoded() : cost.demand()))
+            break;
+        const int rc = decode ? launch_render_decoded(s, d_uv, d_disp, out_w, out_h, n, d_out, st, d_out8)
+                              : launch_render_demand(s, d_uv, d_disp, out_w, out_h, n, d_out, st, d_out8);
         if (rc != RLFC_E_UNSUPPORTED)
             return rc;
     }
