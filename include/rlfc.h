@@ -168,7 +168,9 @@ RLFC_API int rlfc_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, co
  * of them, and about 200 bytes per camera); if that allocation fails the
  * call decodes on demand instead.  Outputs much smaller than the views of a
  * large light field (thumbnails) decode just the pixels they sample, without
- * scratch, where that is estimated to be the faster.  The loaded stream's own memory pool keeps
+ * scratch, where that is estimated to be the faster.  Under stream capture
+ * only calls of four or more cameras at the views' own size allocate, so the
+ * graphs of all others hold no memory nodes.  The loaded stream's own memory pool keeps
  * what its calls used for the next ones, up to four times the packed size of
  * all its views (64 MiB at least, 4 GiB at most), until rlfc_free_stream.  Results do not depend
  * on the path or on the other views of the call.

@@ -30,6 +30,11 @@ namespace {
 // 5 x 5 x 256^2 34 / 42 (three), 36 / 43 (four), 64 / 49 (eight).
 constexpr uint32_t kDecodeFirstViews = 3;
 constexpr uint64_t kDecodeFirstPixels = 400000;
+// A call under stream capture that allocates makes memory nodes, and a graph
+// with those can be neither a child graph nor instantiated twice.  Only native
+// calls of this many cameras may: the others are captured on demand or pixel
+// by pixel, which need no scratch.
+constexpr uint32_t kCapturedScratchViews = 4;
 
 __constant__ uint32_t c_modes[kNumModes] = RLFC_MODE_TABLE_INIT;
 
@@ -139,18 +144,31 @@ struct Estimate {
     double direct() const { return 90 + nodes * (n < 3 ? 0.7 : 1.5) + px * (700 + 12 * nodes); }
 };
 
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+        cudaGetLastError();   // the legacy stream beside another one's capture: not captured itself
+        return false;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+
 }  // namespace
 
 int launch_render(const rlfc_stream *s, const float *d_uv, const float *d_disp, uint32_t out_w,
                   uint32_t out_h, uint32_t n, float *d_out, cudaStream_t st, uint8_t *d_out8)
 {
-    const bool first = n >= kDecodeFirstViews && (uint64_t)n * s->info.W * s->info.H >= kDecodeFirstPixels;
     const bool native = out_w == s->info.W && out_h == s->info.H;
+    const bool scratch = (native && n >= kCapturedScratchViews) || !capturing(st);
+    const bool first = scratch && n >= kDecodeFirstViews && (uint64_t)n * s->info.W * s->info.H >= kDecodeFirstPixels;
     const Estimate cost(*s, out_w, out_h, n);
     for (int turn = 0; turn < 2; turn++) {
         // the other path where the first cannot run: no scratch to decode
         // into, or a tile's footprint too large for shared memory
         const bool decode = (turn == 0) == first;
+        if (decode && !scratch)
+            continue;
         if (!native && cost.direct() < 0.95 * (decode ? cost.decoded() : cost.demand()))
             break;
         const int rc = decode ? launch_render_decoded(s, d_uv, d_disp, out_w, out_h, n, d_out, st, d_out8)
