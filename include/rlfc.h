@@ -170,10 +170,11 @@ RLFC_API int rlfc_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, co
  * large light field (thumbnails) decode just the pixels they sample, without
  * scratch, where that is estimated to be the faster.  Under stream capture
  * only calls of four or more cameras at the views' own size allocate, so the
- * graphs of all others hold no memory nodes.  The loaded stream's own memory pool keeps
- * what its calls used for the next ones, up to four times the packed size of
- * all its views (64 MiB at least, 4 GiB at most), until rlfc_free_stream.  Results do not depend
- * on the path or on the other views of the call.
+ * graphs of all others hold no memory nodes.  The loaded
+ * streams of a device share a memory pool, which keeps what their calls used
+ * for the next ones: up to four times the packed size of all their views (64
+ * MiB at least, 4 GiB at most, in all), until they are freed.  Results do
+ * not depend on the path or on the other views of the call.
  * Errors: RLFC_E_INVALID_ARG, RLFC_E_RANGE, RLFC_E_UNSUPPORTED, RLFC_E_CUDA.
  */
 RLFC_API int rlfc_render_views(const rlfc_stream *s, const float *d_uv, const float *d_disp,

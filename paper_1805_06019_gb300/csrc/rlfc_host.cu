@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -283,6 +284,83 @@ int parse(const uint8_t *p, size_t n, Parsed &ps)
     return RLFC_OK;
 }
 
+// The scratch pool of a device, shared by the light fields loaded on it: it
+// keeps what render calls used for the next ones, up to four calls' largest
+// scratch (the packed views of the whole light field) of every loaded light
+// field, within these bounds in all; a freed light field takes its part with
+// it, the last one the pool.  (The device's default pool gives everything back
+// at each synchronisation: a call after one then maps its memory anew, 180 us
+// for one view and 400 us for 85 MB.  A bound below what the calls in flight
+// on a server's four streams hold does the same to them: at 80 000 small views
+// per second 0.8 ms of latency instead of 0.1.  A pool per light field kept as
+// much again for each: 24 of 5 x 5 x 352^2 rendered in turn held 768 MiB, the
+// shared pool 32.)
+constexpr uint64_t kScratchKeepLeast = 64ull << 20, kScratchKeepMost = 4ull << 30;
+
+struct ScratchPool {
+    cudaMemPool_t pool;
+    uint64_t keep;      // sum over the loaded light fields
+    uint32_t streams;   // loaded light fields that use it
+};
+constexpr int kMaxDevices = 64;
+ScratchPool g_pools[kMaxDevices];
+std::mutex g_pools_lock;
+
+uint64_t scratch_keep(const rlfc_stream &s)
+{
+    return 4 * (4ull * packed_pitch(s.info.W) * s.info.H * s.tab.n_views + (1u << 20));
+}
+
+cudaError_t bound_pool(ScratchPool &p)
+{
+    uint64_t keep = std::clamp<uint64_t>(p.keep, kScratchKeepLeast, kScratchKeepMost);
+    return cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+void join_pool(rlfc_stream *s)
+{
+    if (s->device < 0 || s->device >= kMaxDevices)
+        return;   // render calls then use the default pool
+    std::lock_guard<std::mutex> lock(g_pools_lock);
+    ScratchPool &p = g_pools[s->device];
+    if (p.streams == 0) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = s->device;
+        p.keep = 0;
+        if (cudaMemPoolCreate(&p.pool, &props) != cudaSuccess || bound_pool(p) != cudaSuccess) {
+            if (p.pool)
+                cudaMemPoolDestroy(p.pool);
+            p.pool = nullptr;
+            cudaGetLastError();
+            return;
+        }
+    }
+    p.streams++;
+    p.keep += scratch_keep(*s);
+    bound_pool(p);
+    s->pool = p.pool;
+}
+
+void leave_pool(rlfc_stream *s)
+{
+    if (!s->pool)
+        return;
+    std::lock_guard<std::mutex> lock(g_pools_lock);
+    ScratchPool &p = g_pools[s->device];
+    p.keep -= scratch_keep(*s);
+    if (--p.streams == 0) {
+        cudaMemPoolDestroy(p.pool);
+        p.pool = nullptr;
+    } else {
+        bound_pool(p);
+        cudaMemPoolTrimTo(p.pool, std::clamp<uint64_t>(p.keep, kScratchKeepLeast, kScratchKeepMost));
+    }
+    s->pool = nullptr;
+}
+
 void free_device(rlfc_stream *s)
 {
     cudaFree(s->d_records);
@@ -291,42 +369,13 @@ void free_device(rlfc_stream *s)
     cudaFree(s->d_node_info);
     cudaFree(s->d_view_anc);
     cudaFree(s->d_debug);
+    leave_pool(s);
     s->d_debug = nullptr;
-    if (s->pool)
-        cudaMemPoolDestroy(s->pool);
-    s->pool = nullptr;
     s->d_records = nullptr;
     s->d_offsets = nullptr;
     s->d_top = nullptr;
     s->d_node_info = nullptr;
     s->d_view_anc = nullptr;
-}
-
-// The pool keeps what render calls used for the next ones: up to four calls'
-// largest scratch (the packed views of the whole light field each), within
-// these bounds.  (The device's default pool gives everything back at each
-// synchronisation: a call after one then maps its memory anew, 180 us for one
-// view and 400 us for 85 MB.  A bound below what the calls in flight on a
-// server's four streams hold does the same to them: at 80 000 small views per
-// second 0.8 ms of latency instead of 0.1.)
-constexpr uint64_t kScratchKeepLeast = 64ull << 20, kScratchKeepMost = 4ull << 30;
-
-void make_pool(rlfc_stream *s)
-{
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.handleTypes = cudaMemHandleTypeNone;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = s->device;
-    const uint64_t call = 4ull * packed_pitch(s->info.W) * s->info.H * s->tab.n_views + (1u << 20);
-    uint64_t keep = std::clamp<uint64_t>(4 * call, kScratchKeepLeast, kScratchKeepMost);
-    if (cudaMemPoolCreate(&s->pool, &props) != cudaSuccess ||
-        cudaMemPoolSetAttribute(s->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        if (s->pool)
-            cudaMemPoolDestroy(s->pool);
-        s->pool = nullptr;   // render calls then use the default pool
-        cudaGetLastError();
-    }
 }
 
 int load(const uint8_t *bytes, size_t nbytes, cudaStream_t st, rlfc_stream **out)
@@ -416,7 +465,7 @@ int load(const uint8_t *bytes, size_t nbytes, cudaStream_t st, rlfc_stream **out
             return RLFC_E_UNSUPPORTED;
         }
     }
-    make_pool(s);
+    join_pool(s);
     *out = s;
     return RLFC_OK;
 }

@@ -47,7 +47,7 @@ struct rlfc_stream {
     int16_t *d_top = nullptr;        // [n_top][nloc][3][16], block-major YCoCg-R
     uint32_t *d_node_info = nullptr; // [S]
     uint32_t *d_view_anc = nullptr;  // [n_views][kMaxLevels]
-    cudaMemPool_t pool = nullptr;    // stream-ordered scratch of render calls (null: the device's default pool)
+    cudaMemPool_t pool = nullptr;    // stream-ordered scratch of render calls, shared by the device's light fields (null: its default pool)
     uint32_t *d_debug = nullptr;     // debug builds: the bounds checks' flag word (rlfc_debug_flags)
 };
 
@@ -108,7 +108,7 @@ int launch_decode_packed(const rlfc_stream *s, uint32_t *d_out, const uint8_t *n
 int block_magnitude(const rlfc_stream *s, cudaStream_t st, uint32_t *mag);
 int launch_decode_blocks(const rlfc_stream *s, const uint32_t *d_view, const uint32_t *d_loc,
                          uint32_t n, uint8_t *d_out, uint8_t *d_status, cudaStream_t st);
-// Stream-ordered scratch for one call, from the stream's own pool (released
+// Stream-ordered scratch for one call, from the device's scratch pool (released
 // with cudaFreeAsync).
 cudaError_t scratch_alloc(const rlfc_stream *s, void **p, size_t bytes, cudaStream_t st);
 // n views (d_out8: when set, 8-bit RGB instead of d_out) from views decoded
