@@ -526,11 +526,8 @@ bool scratch_bounds(const rlfc_enc_params *p, uint64_t &fixed, uint64_t &records
             add(2 * npix * cnt[l]);
         if (l + 1 < L)
             add(cnt[l] * 3 * nloc);
-        if (l + 1 < L)
-            add(cnt[l] * 3 * nloc);
     }
     add(sizeof(int));
-    add(sizeof(void *) * L);
     for (uint32_t l = 1; l < L; l++) {
         add(4 * (cnt[l] + 1));
         add(4 * cnt[l - 1]);
@@ -542,7 +539,6 @@ bool scratch_bounds(const rlfc_enc_params *p, uint64_t &fixed, uint64_t &records
     add(4 * S);
     add(4 * 3 * nloc);
     add(4 * (3 * nloc + 1));
-    add(sizeof(int));
     add(sizeof(void *) * L);
     add(sizeof(void *) * L);
     const uint64_t MW = (S + 31) / 32;
