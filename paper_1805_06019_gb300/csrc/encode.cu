@@ -131,7 +131,7 @@ struct SrvArgs {
     int16_t *leaf_resid;      // level 0 only, may be null: residuals after the pixel threshold
     uint8_t *leaf_label;      // level 0 only, may be null: search result, 0xFF = not kept
     int *error;
-    uint32_t n_child, nlx, nloc, Wp, Hp;
+    uint32_t nlx, nloc, Wp, Hp;
     int32_t tau_p, tau_b;
     uint32_t q;
     uint32_t mode_space, lam_q8;
@@ -710,7 +710,6 @@ int encode_gpu(const rlfc_enc_params *p, const uint8_t *d_rgb, cudaStream_t st, 
         s.mode_space = p->mode_space;
         s.lam_q8 = p->lam_q8;
         s.tau_err = p->tau_err;
-        s.n_child = cnt[l - 1];
         s.nlx = nlx;
         s.nloc = nloc;
         s.Wp = Wp;

@@ -330,6 +330,10 @@ int launch_render_demand(const rlfc_stream *s, const float *d_uv, const float *d
     // views are small, still makes two CTAs per SM; a footprint too large for
     // that takes the smallest tile
     static const int tiles[][2] = {{32, 16}, {32, 8}, {16, 8}, {8, 8}};
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "render_demand: SM count");
     uint32_t smem = 0;
     for (const auto &t : tiles) {
         a.tx = t[0];
@@ -345,14 +349,13 @@ int launch_render_demand(const rlfc_stream *s, const float *d_uv, const float *d
         smem = (uint32_t)std::min<uint64_t>(need, UINT32_MAX);
         a.tiles_x = (out_w + t[0] - 1) / t[0];
         const uint64_t ctas = (uint64_t)a.tiles_x * ((out_h + t[1] - 1) / t[1]) * n;
-        if (smem <= kSmemFourCtas && ctas >= 2 * 152)
+        if (smem <= kSmemFourCtas && ctas >= 2 * (uint64_t)sms)
             break;
     }
     const uint64_t n_tiles = (uint64_t)a.tiles_x * ((out_h + a.ty - 1) / a.ty);
     if (smem > kSmemMost || n_tiles >= (1ull << 31))
         return RLFC_E_UNSUPPORTED;
     auto kern = native ? render_demand_kernel<true> : render_demand_kernel<false>;
-    cudaError_t e;
     // (the same limit for every call: the attribute belongs to the kernel, and
     // a smaller one set for another thread's light field would refuse this launch)
     if (smem > 40u * 1024u && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost)) != cudaSuccess)
