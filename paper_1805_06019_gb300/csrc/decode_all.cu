@@ -652,10 +652,10 @@ int launch_decode(const rlfc_stream *s, uint8_t *d_out, const uint8_t *needed, c
     // of most strips fit a third of its shared memory, else two of twelve:
     // set-up, parse and internal nodes wait on memory and barriers, and more
     // CTAs overlap them with the view work of the others.  Measured, three
-    // against two: 9 x 9 x 512^2 75 / 83 us, 32 of its views packed 64 / 70,
-    // 5 x 5 x 64^2 16.8 / 17.4; 17 x 17 x 1024^2, whose records then read
-    // from the stream, 706 / 693.  Strips whose records do not fit what is
-    // left read them from the stream.
+    // against two: 9 x 9 x 512^2 (12 MB stream) 75 / 83 us, 32 of its views
+    // packed 64 / 70, 5 x 5 x 64^2 16.8 / 17.4; 17 x 17 x 1024^2 (133 MB
+    // stream), whose records then read from the stream, 706 / 693.  Strips
+    // whose records do not fit what is left read them from the stream.
     const uint32_t strips = (a.nlx + kNL - 1) / kNL * s->info.nloc_y;
     const size_t longest = 4ull * ((s->max_strip_words + 8 + 3 + 3) & ~3u);
     const size_t most = std::min<size_t>(longest, 4ull * (s->record_words / strips) * 3 / 2 + 64);

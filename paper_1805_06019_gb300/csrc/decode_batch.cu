@@ -25,9 +25,10 @@
 //
 // What bounds it: the chain of dependent loads per location and instruction
 // issue (57 % of the slots, 27 of 32 lanes active); 10^6 requests on the 17 x
-// 17 x 1024^2 light field (133 MB stream) take 0.189 ms, 0.15 of them here.
-// With 32-bit accumulators, an atomic per value, the sequential bit reader,
-// eight requests a round and one record parsed after the other: 0.323 ms.
+// 17 x 1024^2 light field take 0.198 ms (133 MB stream) or 0.183 (99 MB, L2
+// flushed; timed one by one 0.155 here, 0.045 the binning).  With 32-bit
+// accumulators, an atomic per value, the sequential bit reader, eight requests
+// a round and one record parsed after the other: 0.338 ms (133 MB).
 #include <cuda_runtime.h>
 
 #include <cuda_pipeline.h>

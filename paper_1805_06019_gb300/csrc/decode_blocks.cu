@@ -15,7 +15,8 @@ namespace {
 constexpr int kWarpsPerCta = 8;
 // The thread-per-channel form pays from this many requests on (fewer leave its
 // long walks with too little to overlap), more for records of many nodes.
-// Measured, a warp per request / a thread per channel, us: 9 x 9 views (three
+// Measured, a warp per request / a thread per channel, us of queued calls (of
+// the 10.4 at 4096 requests the kernel takes 9.2): 9 x 9 views (three
 // mask words) 10.4 / 14.8 at 4096, 14.6 / 14.6 at 8192, 98 / 33 at 10^5; 17 x
 // 17 views (ten words) 16.7 / 24.7 at 8192, 24.8 / 24.8 at 16384, 103 / 55 at
 // 10^5; 5 x 5 views 10.0 / 9.2 at 4096, 103 / 21 at 10^5.

@@ -189,9 +189,10 @@ __device__ __forceinline__ void row_to_rgb(const uint2 y, const uint2 co, const 
 // neighbouring strips, go out in smaller pieces.
 //
 // What bounds it: instruction issue (about 25 instructions for up to 512
-// bytes; the edges another 30).  The 15 x 15 x 625 x 434 decode takes 0.249 ms
-// with it; with single bytes or 4-byte words, each placed by divisions by the
-// row length, it took 0.695 ms; with the edges as single bytes, 0.255.
+// bytes; the edges another 30).  The 15 x 15 x 625 x 434 decode (31 MB stream)
+// takes 0.246 ms with it; with single bytes or 4-byte words, each placed by
+// divisions by the row length, it took 0.706 ms; with the edges as single
+// bytes, 0.255.
 __device__ __forceinline__ void store_row_unaligned(uint8_t *row, const uint32_t *src, uint32_t len, uint32_t ch)
 {
     const int b0 = (int)(16u * ch) - (int)((uintptr_t)row & 15u);

@@ -24,10 +24,13 @@ namespace {
 // Calls of at least this many cameras over at least this many source pixels
 // decode the neighbour views they need first (one pass over every record,
 // then a cheap blend per camera); smaller ones decode tile by tile on demand,
-// which costs more per camera but touches only what a camera sees.  Measured,
-// on demand / decoded first, us: 9 x 9 x 512^2 44 / 75 (one camera), 73 / 80
-// (two), 114 / 82 (three); 17 x 17 x 1024^2 214 / 359, 345 / 376, 575 / 398;
-// 5 x 5 x 256^2 34 / 42 (three), 36 / 43 (four), 64 / 49 (eight).
+// which costs more per camera but touches only what a camera sees.  Measured at
+// the views' own size, on demand / decoded first, us of queued calls: 9 x 9 x
+// 512^2 27 / 58 (one camera), 47 / 65 (two), 70 / 68 (three), 90 / 73 (four);
+// 17 x 17 x 1024^2 126 / 374, 205 / 393, 370 / 421, 492 / 441; 15 x 15 x 625 x
+// 434 36 / 109, 58 / 117, 100 / 126, 134 / 134; 5 x 5 x 256^2 23 / 33 (three),
+// 27 / 35 (four), 45 / 39 (eight).  So the line lies between three and four
+// cameras; three on the larger fields are up to a quarter slower for it.
 constexpr uint32_t kDecodeFirstViews = 3;
 constexpr uint64_t kDecodeFirstPixels = 400000;
 // A call under stream capture that allocates makes memory nodes, and a graph

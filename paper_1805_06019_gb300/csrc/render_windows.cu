@@ -13,7 +13,7 @@
 //     shifted windows fit shared memory, marks the views needed and numbers
 //     their slots;
 //  2. the needed views are decoded into packed RGB slots (decode_all.cu);
-//  3. render_native_kernel: persistent CTAs take (group, 64 x 32 tile) items
+//  3. render_native_kernel: persistent CTAs take (group, 64 x 16 tile) items
 //     from a queue, fill one window of the tile per neighbour, and blend the
 //     group's cameras from the windows.
 #include <cuda_runtime.h>
