@@ -317,6 +317,14 @@ cudaError_t bound_pool(ScratchPool &p)
     return cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
 }
 
+// A bound that could not be changed leaves the old one, and no error behind
+// for the next launch to find.
+void settle(cudaError_t e)
+{
+    if (e != cudaSuccess)
+        cudaGetLastError();
+}
+
 void join_pool(rlfc_stream *s)
 {
     if (s->device < 0 || s->device >= kMaxDevices)
@@ -340,7 +348,7 @@ void join_pool(rlfc_stream *s)
     }
     p.streams++;
     p.keep += scratch_keep(*s);
-    bound_pool(p);
+    settle(bound_pool(p));
     s->pool = p.pool;
 }
 
@@ -355,8 +363,8 @@ void leave_pool(rlfc_stream *s)
         cudaMemPoolDestroy(p.pool);
         p.pool = nullptr;
     } else {
-        bound_pool(p);
-        cudaMemPoolTrimTo(p.pool, std::clamp<uint64_t>(p.keep, kScratchKeepLeast, kScratchKeepMost));
+        settle(bound_pool(p));
+        settle(cudaMemPoolTrimTo(p.pool, std::clamp<uint64_t>(p.keep, kScratchKeepLeast, kScratchKeepMost)));
     }
     s->pool = nullptr;
 }
